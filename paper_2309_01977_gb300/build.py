@@ -18,8 +18,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libspect.so")
 SOURCES = ["spect_api.cu", "plane_host.cu", "gather_kernel.cu", "gather_tiled.cu", "misc_kernels.cu",
-           "forward_ipt1.cu", "forward_ipt2.cu", "forward_ipt3.cu", "forward_ipt4.cu",
-           "blur_back_ipt1.cu", "blur_back_ipt2.cu", "blur_back_ipt3.cu", "blur_back_ipt4.cu",
+           "forward_1.cu", "forward_2.cu", "forward_3.cu", "forward_4.cu", "forward_5.cu",
+           "blur_back_1.cu", "blur_back_2.cu", "blur_back_3.cu", "blur_back_4.cu",
            "noalloc.cu", "psf_bf16.cu", "serve.cu", "pet.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -88,4 +88,10 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// The same for the 128-byte line at p (any address), as a per-lane request.
+__device__ __forceinline__ void prefetch_line_l2(const void* p)
+{
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory");
+}
+
 }  // namespace spect

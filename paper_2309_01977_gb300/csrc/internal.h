@@ -17,8 +17,10 @@ namespace spect {
 
 constexpr int kMaxR = 20;            // largest supported PSF radius (taps 2*kMaxR+1)
 constexpr int kTapW = 2 * kMaxR + 1; // row width of the device taps table
+constexpr int kLowR = 14;            // largest radius of the plane kernels' narrow variants
+constexpr int kTapRow = kMaxR + 1;   // floats of a shared-memory row of taps w(0..kMaxR)
 constexpr int kStrip = 16;           // outputs per thread along one blur strip
-constexpr int kFwdThreads = 512;     // most threads of the forward / blur kernels
+constexpr int kPlaneThreads = 512;   // most threads of the FP32 forward / back blur kernels
 constexpr int kMaxCand = 9;          // rotated-grid samples that can touch one voxel
 constexpr int kMaxIpt = 4;           // largest j-blur strips per thread
 constexpr int kTcTile = 128 * 128;   // BF16 Toeplitz tile, elements
@@ -44,14 +46,35 @@ struct PlaneTiling {
     int sq;       // Q stride between column pairs, in quads (odd): >= (npad + 2*rh) / 2
     int threads;  // CTA size (multiple of 32, <= kFwdThreads)
     int ipt;      // j-blur strips per thread (1..kMaxIpt)
-    size_t smem;  // P, Q, the forward's tap-row table and the tap buffer, bytes
-    // Attenuation planes staged in shared memory by bulk copies, one plane
-    // ahead: row width in floats (0 when the buffer does not fit and A is
-    // read from global memory), and byte offsets of the tap buffer, the
-    // attenuation buffer and its mbarrier; per kernel (f: forward, b: back).
-    int a_cols_f, off_taps_f, off_a_f, off_bar_f;
-    int a_cols_b, off_taps_b, off_a_b, off_bar_b;
-    size_t smem_f, smem_b;  // dynamic shared memory of each kernel
+    bool high;    // radii past kLowR, or several strips per thread: the kernel with every radius
+    // Attenuation planes staged in shared memory by one bulk copy each, a
+    // plane ahead (else A is read from global memory); byte offsets of the tap
+    // buffer, the attenuation buffer and its mbarrier.
+    bool smem_a;
+    int off_taps, off_a, off_bar;
+    size_t smem;  // dynamic shared memory: P, Q, the tap-row table, the tap buffer, the attenuation buffer
+};
+
+// Shape of one back blur launch (blur_back.cuh).
+constexpr int kBackStrides[] = {9, 17, 33, 49, 65};  // strides of Q: half a tile's columns, rounded up to odd
+
+// threads % width and threads / width of a grid of items, `width` to a row.
+struct ItemStep {
+    int dc, dr;
+};
+
+struct BackTiling {
+    int ktile, ntiles;  // as above
+    int rh;             // halo = largest PSF radius, rounded up to even
+    int ktpad, npad;
+    int sp, sq;         // strides between row pairs of the projection (odd) and of Q (one of kBackStrides), in quads
+    int pad_rows;       // zero row pairs above and below Q
+    int threads;
+    ItemStep zstep, jstep;  // of the z-blur (row pairs to a row) and j-blur strips (column pairs to a row)
+    bool smem_a;        // A_i staged in shared memory by bulk copies, one plane ahead; else read from global memory
+    bool high;          // radii past kLowR
+    int off_q, off_taps, off_a, off_bar;
+    size_t smem;        // dynamic shared memory
 };
 
 struct ForwardArgs {
@@ -104,7 +127,7 @@ struct BlurBackArgs {
     const int* sel;        // [n_sel] angle ids
     int n, nz, n_sel, batch;
     int chunks;            // depth chunks: contiguous plane ranges of equal work
-    PlaneTiling t;
+    BackTiling t;
     float* bvol;           // [batch][n_sel][n][n][nz] rotated-frame volumes A . (K_i r)
     int* err;              // SPECT_ETIMEDOUT when a bounded wait runs out
 };
@@ -206,20 +229,22 @@ uint32_t bf16_tmem_cols(int n, int tiles);  // TMEM columns: `tiles` n-column ac
 int bf16_occupancy(int n);
 
 PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit);
-cudaError_t launch_forward(const ForwardArgs& a, int grid_x, cudaStream_t st);
-cudaError_t launch_blur_back(const BlurBackArgs& a, int grid_x, cudaStream_t st);
+BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit);
+cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t st);
+cudaError_t launch_blur_back(const BlurBackArgs& a, cudaStream_t st);
+int forward_max_blocks_per_sm(const PlaneTiling& t);
+int blur_back_max_blocks_per_sm(const BackTiling& t);
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t st);
 cudaError_t launch_gather_tables(const float4* cs, int n, int nz, int n_angles, int2* tab, cudaStream_t st);
 cudaError_t launch_gather_tiled_tables(const float4* cs, int n, int nz, int n_angles, int T, int2* tab, int* desc,
                                        int* rows_max, int* err, cudaStream_t st);
 cudaError_t launch_gather_tiled(const GatherTiledArgs& a, cudaStream_t st);
 size_t gather_tiled_smem(int rows_cap, int zs, int T, int stages, int n_sel);  // n_sel: angles per launch
-int forward_max_blocks_per_sm(const PlaneTiling& t);
-
-// Per-IPT instantiations (one translation unit each, compiled in parallel).
-template <int IPT> cudaError_t forward_launch_ipt(const ForwardArgs& a, int grid_x, cudaStream_t st);
-template <int IPT> int forward_occupancy_ipt(int threads, size_t smem);
-template <int IPT> cudaError_t blur_back_launch_ipt(const BlurBackArgs& a, int grid_x, cudaStream_t st);
+// Instantiations compiled in translation units of their own.
+template <int IPT, bool kHigh> cudaError_t forward_launch_ipt(const ForwardArgs& a, cudaStream_t st);
+template <int IPT, bool kHigh> int forward_occupancy_ipt(int threads, size_t smem);
+template <bool kSmemA, bool kHigh> cudaError_t launch_blur_back_v(const BlurBackArgs& a, cudaStream_t st);
+template <bool kSmemA, bool kHigh> int blur_back_blocks_v(const BackTiling& t);
 
 // misc kernels
 cudaError_t launch_attenuation(const float* mu, const float4* cs, int n, int nz, int n_angles,
@@ -269,7 +294,8 @@ struct spect_plan {
     int psf_tables = 1;                     // PSF tables: n_angles for a non-circular orbit, else 1
     int max_subset = 0;
     spect::PlaneTiling tiling{};
-    int fwd_occ = 1;         // resident forward CTAs per SM
+    spect::BackTiling back{};
+    int fwd_occ = 1, back_occ = 1;  // resident forward / back blur CTAs per SM
 
     // device memory
     float4* d_cs = nullptr;                   // [na] (cos, sin, cj = c + T_trans shift, 0)

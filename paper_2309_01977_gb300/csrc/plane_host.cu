@@ -1,4 +1,4 @@
-// Host-side tiling and dispatch of the plane-blur kernels.
+// Host-side tiling and dispatch of the FP32 plane kernels.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -7,69 +7,56 @@
 
 namespace spect {
 
-static int round_up(int v, int m) { return (v + m - 1) / m * m; }
+namespace {
 
-static PlaneTiling make_tiling(int n, int nz, int rmax, int ktile)
+int round_up(int v, int m) { return (v + m - 1) / m * m; }
+
+constexpr size_t kSmSmem = 228 * 1024;  // shared memory of an SM; each resident CTA takes 1 KB on top of its own
+
+// Forward z tile of ktile columns; smem 0 where its strips do not fit.
+PlaneTiling make_tiling(int n, int nz, int rmax, int ktile, size_t cap, size_t limit)
 {
     PlaneTiling t{};
     t.ktile = ktile;
     t.ntiles = (nz + ktile - 1) / ktile;
-    t.rh = rmax + (rmax & 1);
+    // even; a multiple of 4 keeps the staged window of a tile 16-byte aligned
+    t.rh = round_up(rmax, t.ntiles > 1 ? 4 : 2);
     t.ktpad = round_up(ktile, kStrip);
     t.npad = round_up(n, kStrip);
     t.sp = ((t.ktpad + 2 * t.rh) / 2) | 1;
     t.sq = ((t.npad + 2 * t.rh) / 2) | 1;
-    // j-blur strips: ktpad/2 column pairs x npad/kStrip row strips; the
-    // smallest number of strips per thread that fits in kFwdThreads threads
-    const int items = (t.ktpad / 2) * (t.npad / kStrip);
-    t.ipt = kMaxIpt + 1;
-    for (int ipt = 1; ipt <= kMaxIpt; ++ipt) {
-        const int thr = round_up((items + ipt - 1) / ipt, 32);
-        if (thr <= kFwdThreads) {
-            t.ipt = ipt;
-            t.threads = std::max(64, thr);
-            break;
-        }
-    }
-    // P and Q quads, the forward's per-plane tap-row table (32 bytes per
-    // row) and the two-plane tap buffer
+    // P and Q quads, the per-plane tap-row table (32 bytes per row) and the
+    // two-plane tap buffer
     const size_t pq = 16 * ((size_t)(t.npad / 2) * t.sp + (size_t)(t.ktpad / 2) * t.sq);
-    const size_t taps = 2 * (kMaxR + 1) * sizeof(float);
-    t.smem = pq + 32 * (size_t)n + taps;
-    t.off_taps_f = (int)(pq + 32 * (size_t)n);
-    t.off_taps_b = (int)pq;
-    t.smem_f = t.smem;
-    t.smem_b = pq + taps;
+    t.off_taps = (int)(pq + 32 * (size_t)n);
+    t.smem = (size_t)t.off_taps + 2 * kTapRow * sizeof(float);
+    // the attenuation buffer where it fits and a plane is one copy (a tile's
+    // rows would be copied one by one, about 60 ns each)
+    const size_t off = (t.smem + 15) & ~(size_t)15, end = off + (size_t)n * nz * sizeof(float);
+    if (t.ntiles == 1 && end + 8 <= limit) {
+        t.smem_a = true;
+        t.off_a = (int)off;
+        t.off_bar = (int)end;
+        t.smem = end + 8;
+    }
+    // CTA size.  The staging and its latency scale with the warps, so a CTA
+    // takes all the threads an SM holds, or half of them where two fit: at
+    // least a thread per j-blur strip (ktpad/2 column pairs x npad/kStrip row
+    // strips) where that is within the limit, else several strips per thread.
+    // Measured (forward, one subset): 64^3 x 8 angles 4 x 128 threads 18.5 us,
+    // 2 x 256 16.5, 1 x 512 18.4; 96^3 x 12 288 threads 48.9, 512 45.2;
+    // 132 x 44 x 60 2 x 224 242, 1 x 320 375, 1 x 448 347.
+    const int items = (t.ktpad / 2) * (t.npad / kStrip);
+    const bool two = 2 * (t.smem + 1024) <= kSmSmem;
+    t.threads = two && items <= kPlaneThreads / 2 ? kPlaneThreads / 2 : kPlaneThreads;
+    t.ipt = (items + t.threads - 1) / t.threads;
+    t.high = rmax > kLowR || t.ipt > 1;
+    if (t.ipt > kMaxIpt || (size_t)t.off_taps + 2 * kTapRow * sizeof(float) > cap) t.smem = 0;
     return t;
 }
 
-// Attenuation buffers of one plane (rows of the columns a CTA reads: the
-// staged window for the forward, the tile for the back blur, widened to
-// 16-byte boundaries), where they fit under `limit` bytes.
-static void attach_atten_buffers(PlaneTiling& t, int n, int nz, size_t limit)
-{
-    const int win = t.ktpad + 2 * t.rh;
-    const int cols_f = t.ntiles == 1 ? nz : std::min(nz, round_up(win + 3, 4));
-    const int cols_b = t.ntiles == 1 ? nz : t.ktile;
-    const size_t off_f = (t.smem_f + 15) & ~(size_t)15, off_b = (t.smem_b + 15) & ~(size_t)15;
-    const size_t end_f = off_f + (size_t)n * cols_f * sizeof(float), end_b = off_b + (size_t)n * cols_b * sizeof(float);
-    t.a_cols_f = t.a_cols_b = 0;
-    if (end_f + 8 <= limit) {
-        t.a_cols_f = cols_f;
-        t.off_a_f = (int)off_f;
-        t.off_bar_f = (int)end_f;
-        t.smem_f = end_f + 8;
-    }
-    if (end_b + 8 <= limit) {
-        t.a_cols_b = cols_b;
-        t.off_a_b = (int)off_b;
-        t.off_bar_b = (int)end_b;
-        t.smem_b = end_b + 8;
-    }
-}
-
 // Columns of the volume a tiling stages per plane (tile plus in-volume halo).
-static long staged_columns(const PlaneTiling& t, int nz)
+long staged_columns(const PlaneTiling& t, int nz)
 {
     long cols = 0;
     for (int tile = 0; tile < t.ntiles; ++tile) {
@@ -79,61 +66,118 @@ static long staged_columns(const PlaneTiling& t, int nz)
     return cols;
 }
 
-// Among the z tilings whose buffers fit `cap`: the one that stages the
-// fewest volume columns per plane (halo columns are staged once per tile),
-// then the fewest j-blur strips (16 column pairs) per thread (each strip per
-// thread repeats the unrolled blur code and its 32 accumulators).  At 192^3
-// (PSF radius 19) two 96-column tiles with two strips per thread beat three
-// 64-column tiles with one: back blur 2.15 vs 4.16 ms, forward 28.2 vs
-// 30.4 ms per batch-of-4 launch on GB300.  Then the attenuation buffers,
-// where they fit under `limit`.
+}  // namespace
+
+// Among the z tilings whose buffers fit `cap`: the one that stages the fewest
+// volume columns per plane (halo columns are staged once per tile), a tiling
+// with several j-blur strips per thread counted half as much again (each
+// strip repeats the unrolled blur code with few warps to hide its latency).
+// At 192^3 (PSF radius 19) three 64-column tiles with 512 threads beat two
+// 96-column tiles with two strips per thread: 1.25 vs 1.51 ms (384 threads)
+// and 1.77 ms (288) per launch of 16 angles and two volumes; at 160^3 two
+// 80-column tiles beat three of 64, 172 vs 233 us for 8 angles.
 PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit)
 {
     PlaneTiling best{};
-    long best_cols = 0;
+    double best_cost = 0;
     for (int nt = 1; nt <= (nz + kStrip - 1) / kStrip; ++nt) {
         const int kt = nt == 1 ? nz : round_up((nz + nt - 1) / nt, kStrip);
         if (nt > 1 && (nt - 1) * kt >= nz) continue;  // same as a smaller count
-        PlaneTiling t = make_tiling(n, nz, rmax, kt);
-        if (t.smem > cap || t.ipt > kMaxIpt) continue;
-        const long cols = staged_columns(t, nz);
-        if (best.smem == 0 || cols < best_cols || (cols == best_cols && t.ipt < best.ipt)) {
+        const PlaneTiling t = make_tiling(n, nz, rmax, kt, cap, limit);
+        if (t.smem == 0) continue;
+        const double cost = (double)staged_columns(t, nz) * (t.ipt > 1 ? 1.5 : 1.0);
+        if (best.smem == 0 || cost < best_cost) {
             best = t;
-            best_cols = cols;
+            best_cost = cost;
         }
     }
-    if (best.smem) attach_atten_buffers(best, n, nz, limit);
+    return best;  // smem == 0: does not fit
+}
+
+// Back blur.  Among the tile widths that fit: the fewest rounds of strips per
+// plane, a CTA of 256 threads (two to an SM) counted half; then the widest
+// tile.  The CTA has 256 threads where a pass over a plane has that many
+// strips or fewer, else 512, and the attenuation comes through shared memory
+// where a tile is the whole plane and the buffer fits.  Measured (one subset,
+// us): 64^3 x 8 angles 256 threads 14.6, two 32-column tiles of 256 16.1;
+// 96^3 x 12 one tile of 512 threads 36.8, two of 256 43.6; 128^3 x 15 one
+// tile of 512 87, two of 256 86; 132 x 44 x 16 256 threads 47.5 (A from global
+// memory 51.3); 160^3 x 8 two tiles of 96 columns 116, five of 32 126; 192^3
+// x 16 x 2 volumes three tiles of 64 columns 332, two of 96 402, six of 32
+// 351; 77 x 77 x 100 x 15 A through shared memory 33.5, from global 65.
+BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit)
+{
+    BackTiling best{};
+    double best_cost = 0.0;
+    const int npad = round_up(n, kStrip), rp = npad / 2, rh = rmax + (rmax & 1);
+    for (int sq : kBackStrides) {
+        BackTiling t{};
+        t.sq = sq;
+        t.ktpad = std::min(2 * (sq - 1), round_up(nz, kStrip));
+        t.ktile = std::min(t.ktpad, nz);
+        t.ntiles = (nz + t.ktile - 1) / t.ktile;
+        t.rh = rh;
+        t.npad = npad;
+        t.pad_rows = (rmax + 1) / 2;
+        t.high = rmax > kLowR;
+        t.sp = ((t.ktpad + 2 * rh) / 2) | 1;
+        size_t off = 16 * (size_t)rp * t.sp;
+        t.off_q = (int)off;
+        off += 16 * (size_t)(rp + 2 * t.pad_rows) * t.sq;
+        t.off_taps = (int)off;
+        off += 2 * kTapRow * sizeof(float);
+        const size_t bare = off, a_at = (off + 15) & ~(size_t)15;  // bulk copies land on 16-byte boundaries
+        const size_t with_a = a_at + (size_t)n * t.ktile * sizeof(float) + 8;
+        t.off_a = (int)a_at;
+        t.off_bar = (int)(with_a - 8);
+        const int zitems = rp * (t.ktpad / kStrip), jitems = (t.ktpad / 2) * (npad / kStrip);
+        t.smem_a = atten && t.ntiles == 1 && with_a <= limit;  // a tile's rows would be copied one by one
+        t.smem = t.smem_a ? with_a : bare;
+        if (t.smem > limit) continue;
+        const int thr = std::max(zitems, jitems) <= kPlaneThreads / 2 ? kPlaneThreads / 2 : kPlaneThreads;
+        t.threads = thr;
+        t.zstep = {thr % rp, thr / rp};
+        t.jstep = {thr % (t.ktpad / 2), thr / (t.ktpad / 2)};
+        const int rounds = (zitems + thr - 1) / thr + (jitems + thr - 1) / thr;
+        const double cost = (double)rounds * thr * t.ntiles;
+        if (best.smem == 0 || cost <= best_cost) {
+            best = t;
+            best_cost = cost;
+        }
+    }
     return best;  // smem == 0: does not fit
 }
 
 int forward_max_blocks_per_sm(const PlaneTiling& t)
 {
     switch (t.ipt) {
-        case 1: return forward_occupancy_ipt<1>(t.threads, t.smem_f);
-        case 2: return forward_occupancy_ipt<2>(t.threads, t.smem_f);
-        case 3: return forward_occupancy_ipt<3>(t.threads, t.smem_f);
-        default: return forward_occupancy_ipt<4>(t.threads, t.smem_f);
+        case 1: return t.high ? forward_occupancy_ipt<1, true>(t.threads, t.smem) : forward_occupancy_ipt<1, false>(t.threads, t.smem);
+        case 2: return forward_occupancy_ipt<2, true>(t.threads, t.smem);
+        case 3: return forward_occupancy_ipt<3, true>(t.threads, t.smem);
+        default: return forward_occupancy_ipt<4, true>(t.threads, t.smem);
     }
 }
 
-cudaError_t launch_forward(const ForwardArgs& a, int grid_x, cudaStream_t st)
+cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t st)
 {
     switch (a.t.ipt) {
-        case 1: return forward_launch_ipt<1>(a, grid_x, st);
-        case 2: return forward_launch_ipt<2>(a, grid_x, st);
-        case 3: return forward_launch_ipt<3>(a, grid_x, st);
-        default: return forward_launch_ipt<4>(a, grid_x, st);
+        case 1: return a.t.high ? forward_launch_ipt<1, true>(a, st) : forward_launch_ipt<1, false>(a, st);
+        case 2: return forward_launch_ipt<2, true>(a, st);
+        case 3: return forward_launch_ipt<3, true>(a, st);
+        default: return forward_launch_ipt<4, true>(a, st);
     }
 }
 
-cudaError_t launch_blur_back(const BlurBackArgs& a, int grid_x, cudaStream_t st)
+int blur_back_max_blocks_per_sm(const BackTiling& t)
 {
-    switch (a.t.ipt) {
-        case 1: return blur_back_launch_ipt<1>(a, grid_x, st);
-        case 2: return blur_back_launch_ipt<2>(a, grid_x, st);
-        case 3: return blur_back_launch_ipt<3>(a, grid_x, st);
-        default: return blur_back_launch_ipt<4>(a, grid_x, st);
-    }
+    if (t.smem_a) return t.high ? blur_back_blocks_v<true, true>(t) : blur_back_blocks_v<true, false>(t);
+    return t.high ? blur_back_blocks_v<false, true>(t) : blur_back_blocks_v<false, false>(t);
+}
+
+cudaError_t launch_blur_back(const BlurBackArgs& a, cudaStream_t st)
+{
+    if (a.t.smem_a) return a.t.high ? launch_blur_back_v<true, true>(a, st) : launch_blur_back_v<true, false>(a, st);
+    return a.t.high ? launch_blur_back_v<false, true>(a, st) : launch_blur_back_v<false, false>(a, st);
 }
 
 }  // namespace spect

@@ -1,6 +1,7 @@
 // C ABI of libspect: plans, forward/back projection, sensitivity, OSEM and
 // the Poisson likelihood.  Host logic only; the kernels live in
-// proj_kernels.cu and misc_kernels.cu.
+// forward.cuh, blur_back.cuh, gather_*.cu and
+// misc_kernels.cu.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -271,9 +272,9 @@ void build_psf(const spect_geom& g, int n, bool psf, double offset, std::vector<
 
 // ---------------------------------------------------------------- launches
 
-int chunk_target(const spect_plan* p, long items)
+int chunk_target(const spect_plan* p, long items, int occ)
 {
-    const long target = (long)p->num_sms * p->fwd_occ;
+    const long target = (long)p->num_sms * occ;
     if (items >= target) return 1;
     return (int)std::max<long>(1, std::min<long>(std::max(1, p->n / 2), target / items));
 }
@@ -288,7 +289,7 @@ int run_forward(spect_plan* p, spect_plan_scratch& sc, const float* x, float* ou
 {
     const PlaneTiling& t = p->tiling;
     // never more chunks than the partial buffer holds for one batch entry
-    const int chunks = (int)std::min<size_t>(chunk_target(p, (long)n_sel * (p->bf16 ? 1 : t.ntiles)),
+    const int chunks = (int)std::min<size_t>(chunk_target(p, (long)n_sel * (p->bf16 ? 1 : t.ntiles), p->fwd_occ),
                                              std::max<size_t>(1, p->partial_planes / (size_t)n_sel));
     // the reduction pass also applies T_fov
     const bool use_partials = chunks > 1 || y != nullptr || p->d_fov != nullptr;
@@ -339,7 +340,7 @@ int run_forward(spect_plan* p, spect_plan_scratch& sc, const float* x, float* ou
             a.out = out + (size_t)b0 * n_sel * plane;
             a.partials = use_partials ? sc.partials : nullptr;
             a.err = p->d_err;
-            e = timed(p, "forward", st, 1, [&] { return launch_forward(a, chunks * t.ntiles, st); });
+            e = timed(p, "forward", st, 1, [&] { return launch_forward(a, st); });
         }
         if (e != cudaSuccess) return cuda_fail(e, "forward kernel launch");
         if (!use_partials) continue;
@@ -398,7 +399,7 @@ int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_
                 bb.nz = p->nz;
                 bb.n_sel = ng;
                 bb.batch = nb;
-                bb.chunks = chunk_target(p, (long)nb * ng);
+                bb.chunks = chunk_target(p, (long)nb * ng, p->back_occ);
                 bb.tmem_cols = bf16_tmem_cols(p->n, 3);  // D1, D2 twice
                 bb.bvol = sc.bvol;
                 bb.err = p->d_err;
@@ -420,12 +421,11 @@ int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_
                 bb.nz = p->nz;
                 bb.n_sel = ng;
                 bb.batch = nb;
-                bb.t = p->tiling;
-                const int chunks = chunk_target(p, (long)nb * ng * p->tiling.ntiles);
-                bb.chunks = chunks;
+                bb.t = p->back;
+                bb.chunks = chunk_target(p, (long)nb * ng * p->back.ntiles, p->back_occ);
                 bb.bvol = sc.bvol;
                 bb.err = p->d_err;
-                e = timed(p, "blur_back", st, 1, [&] { return launch_blur_back(bb, chunks * p->tiling.ntiles, st); });
+                e = timed(p, "blur_back", st, 1, [&] { return launch_blur_back(bb, st); });
             }
             if (e != cudaSuccess) return cuda_fail(e, "blur_back kernel launch");
             if (p->gather_tiled) {
@@ -890,13 +890,19 @@ int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream,
     // leave room for the 1 KB the hardware reserves per CTA and static shared memory
     const size_t cap1 = (size_t)std::min(smem_optin, 227 * 1024) - 2048;
     p->tiling = plane_tiling(p->n, p->nz, p->rmax, cap1, (size_t)smem_optin);
-    if (p->tiling.smem == 0) { free_plan(p); return fail(SPECT_EINVAL, "plane %dx%d too large for shared memory", p->n, p->nz); }
+    p->back = back_tiling(p->n, p->nz, p->rmax, atten, (size_t)smem_optin);
+    if (p->tiling.smem == 0 || p->back.smem == 0) {
+        free_plan(p);
+        return fail(SPECT_EINVAL, "plane %dx%d too large for shared memory", p->n, p->nz);
+    }
     p->bf16 = (g.flags & SPECT_FLAG_PSF_BF16) != 0;
     p->fwd_occ = p->bf16 ? bf16_occupancy(p->n) : std::max(1, forward_max_blocks_per_sm(p->tiling));
+    p->back_occ = p->bf16 ? p->fwd_occ : std::max(1, blur_back_max_blocks_per_sm(p->back));
 
     const size_t vol = vol_elems(p), plane = plane_elems(p);
     const size_t target = (size_t)p->num_sms * p->fwd_occ;
-    p->partial_planes = std::max<size_t>(2 * target, (size_t)p->max_subset);
+    // at most four planes per SM: what a server reserves for a slot
+    p->partial_planes = std::max<size_t>(std::min<size_t>(2 * target, 4 * (size_t)p->num_sms), (size_t)p->max_subset);
     p->bvol_cap = (size_t)std::max(p->max_subset, 16);
     if ((rc = dev_alloc(p, &p->d_cs, p->na)) ||
         (rc = dev_alloc(p, &p->d_taps, taps.size())) ||
