@@ -132,6 +132,19 @@ struct BlurBackArgs {
     int* err;              // SPECT_ETIMEDOUT when a bounded wait runs out
 };
 
+// Back blur of all-ones projections (misc_kernels.cu).
+struct BlurBackOnesArgs {
+    const float* atten;    // [n_angles][n][n][nz] or nullptr
+    const float* taps;
+    const int* rad;
+    size_t taps_stride;    // as ForwardArgs
+    int rad_stride;
+    const int* sel;        // [n_sel] angle ids
+    int n, nz, n_sel;
+    float* bvol;           // [n_sel][n][n][nz]
+};
+cudaError_t launch_blur_back_ones(const BlurBackOnesArgs& a, cudaStream_t st);
+
 // Image update at the end of a subiteration (update.cuh).
 constexpr int kUpdNone = 0, kUpdOsem = 1, kUpdOsl = 2, kUpdBsrem = 3;
 struct UpdateSpec {

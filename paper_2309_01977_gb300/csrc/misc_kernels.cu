@@ -107,6 +107,47 @@ cudaError_t launch_attenuation(const float* mu, const float4* cs, int n, int nz,
     return cudaGetLastError();
 }
 
+// Rotated-frame volumes of all-ones projections (the sensitivities H_m^T 1):
+// the blur of a constant is the outer product of the taps' partial sums at
+// the plane's edges, so B_a[i][j][k] = A_a[i][j][k] v_i(j) w_i(k) with
+// v_i(j) = sum of w_i(t) over 0 <= j - t < n, and w_i(k) alike over nz.  One
+// block per (plane, angle); bound by the HBM traffic of A and B where the
+// blur of every plane was bound by its FMAs (96^3 x 12 angles: see launch).
+__global__ void __launch_bounds__(256) ones_back_kernel(BlurBackOnesArgs a)
+{
+    extern __shared__ float edge[];  // v_i [n], w_i [nz]
+    const int i = blockIdx.x, sidx = blockIdx.y, n = a.n, nz = a.nz;
+    const int angle = a.sel[sidx];
+    const float* taps = a.taps + (size_t)angle * a.taps_stride + (size_t)i * kTapW + kMaxR;
+    const int R = a.rad[(size_t)angle * a.rad_stride + i];
+    for (int e = threadIdx.x; e < n + nz; e += blockDim.x) {
+        const int m = e < n ? n : nz, pos = e < n ? e : e - n;
+        float s = 0.f;
+        for (int t = max(-R, pos - (m - 1)); t <= min(R, pos); ++t) s += __ldg(taps + t);
+        edge[e] = s;
+    }
+    __syncthreads();
+    const int zq = nz >> 2;
+    const float4* A = a.atten ? reinterpret_cast<const float4*>(a.atten + ((size_t)angle * n + i) * n * nz) : nullptr;
+    float4* B = reinterpret_cast<float4*>(a.bvol + ((size_t)sidx * n + i) * n * nz);
+    for (int e = threadIdx.x; e < n * zq; e += blockDim.x) {
+        const int j = e / zq, k = 4 * (e - j * zq);
+        const float v = edge[j];
+        float4 b = make_float4(v * edge[n + k], v * edge[n + k + 1], v * edge[n + k + 2], v * edge[n + k + 3]);
+        if (A) {
+            const float4 q = __ldg(A + e);
+            b = make_float4(b.x * q.x, b.y * q.y, b.z * q.z, b.w * q.w);
+        }
+        B[e] = b;
+    }
+}
+
+cudaError_t launch_blur_back_ones(const BlurBackOnesArgs& a, cudaStream_t st)
+{
+    ones_back_kernel<<<dim3(a.n, a.n_sel), 256, (size_t)(a.n + a.nz) * sizeof(float), st>>>(a);
+    return cudaGetLastError();
+}
+
 // Sum the per-(angle, tile) FP64 partials of one subiteration in a fixed order.
 __global__ void diag_finalize_kernel(const double* __restrict__ part, int n_part, double* __restrict__ out3)
 {

@@ -386,7 +386,20 @@ int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_
         for (int g0 = 0; g0 < n_sel; g0 += G) {
             const int ng = std::min(G, n_sel - g0);
             cudaError_t e;
-            if (p->bf16) {
+            if (!proj && !p->d_fov) {  // all-ones projections (one batch entry)
+                BlurBackOnesArgs bb{};
+                bb.atten = p->d_atten;
+                bb.taps = p->d_taps;
+                bb.rad = p->d_rad;
+                bb.taps_stride = p->psf_tables > 1 ? (size_t)p->n * kTapW : 0;
+                bb.rad_stride = p->psf_tables > 1 ? psf_int_stride(p->n) : 0;
+                bb.sel = sel_dev + g0;
+                bb.n = p->n;
+                bb.nz = p->nz;
+                bb.n_sel = ng;
+                bb.bvol = sc.bvol;
+                e = timed(p, "blur_back_ones", st, 1, [&] { return launch_blur_back_ones(bb, st); });
+            } else if (p->bf16) {
                 BlurBackBf16Args bb{};
                 bb.proj = proj ? proj + ((size_t)b0 * n_sel + g0) * plane : nullptr;
                 bb.proj_bstride = (size_t)n_sel * plane;
