@@ -990,11 +990,19 @@ int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream,
     SPECT_CK(cudaMemcpyAsync(p->d_rad, radw.data(), radw.size() * sizeof(int), cudaMemcpyHostToDevice, st), "copy radii");
     SPECT_CK(cudaMemcpyAsync(p->d_sel_all, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, st), "copy angles");
     // Gather tables.  Tiled (footprints staged in shared memory) for planes
-    // of at least 128 x 128 with nz <= 128 (smaller planes are faster with
-    // the per-column gather): 8 x 8 tiles, whole columns (each run of
-    // footprint rows is one contiguous copy) and two footprint buffers (one
-    // angle in flight; a third buffer measured slower on GB300).
-    p->gather_tiled = p->n >= 128 && p->nz <= 128;
+    // of at least 96 x 96: 8 x 8 tiles, whole columns up to 128 long (each run
+    // of footprint rows is one contiguous copy), longer ones in equal segments
+    // of 80 to 128 where there are such, and two footprint buffers (one angle
+    // in flight; a third buffer measured slower on GB300).  Else the
+    // per-column gather.  Tiled against per column, one subset, us: 64^3 x 8
+    // angles 19.6 / 12.3, 77 x 77 x 100 x 15 33.6 / 33.1, 96^3 x 12 26.7 /
+    // 32.9, 96^3 x 16 x 2 volumes 40.7 / 89.3, 112^3 x 12 31 / 49, 160^3 x 8
+    // (two segments of 80) 89 / 121, 192^3 x 16 (two of 96) 222 / 313, in
+    // three of 64 318.
+    int zs = p->nz <= 128 ? p->nz : 0;
+    for (int d = 2; zs == 0 && p->nz / d >= 80; ++d)
+        if (p->nz % (4 * d) == 0 && p->nz / d <= 128) zs = p->nz / d;
+    p->gather_tiled = p->n >= 96 && zs > 0;
     if (p->gather_tiled) {
         p->gt_T = kGtT;
         const int tx = (p->n + p->gt_T - 1) / p->gt_T;
@@ -1015,7 +1023,7 @@ int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream,
         SPECT_CK(cudaMemcpyAsync(&err, p->d_err, sizeof(int), cudaMemcpyDeviceToHost, st), "read status");
         SPECT_CK(cudaStreamSynchronize(st), "gather tables");
         p->gt_rows = std::max(rows, 1);
-        p->gt_zs = p->nz;
+        p->gt_zs = zs;
         p->gt_stages = 2;
         if (err != 0 || gather_tiled_smem(p->gt_rows, p->gt_zs, p->gt_T, 2, kGatherMaxAngles) > (size_t)smem_optin) {
             // footprints too large for shared memory, or a strip list past
