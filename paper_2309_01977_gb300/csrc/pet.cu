@@ -190,9 +190,10 @@ __device__ __forceinline__ bool walk_setup(const float* __restrict__ lor, const 
 }
 
 // The timing weight of sample i.
-__device__ __forceinline__ float tof_weight(const Walk& k, const TofParams& tp, float cb, const float* tof_tab, int i)
+__device__ __forceinline__ float tof_weight(float l0, float dl, const TofParams& tp, float cb, const float* tof_tab,
+                                            int i)
 {
-    const float x = (fmaf((float)i, k.dl, k.l0) - cb + tp.half_win) * tp.inv_h;
+    const float x = (fmaf((float)i, dl, l0) - cb + tp.half_win) * tp.inv_h;
     const float xc = fminf(fmaxf(x, 0.f), (float)kTofTab);
     const int j = min((int)xc, kTofTab - 1);
     const float fr = xc - (float)j;
@@ -210,7 +211,7 @@ __device__ __forceinline__ void walk(const Walk& k, const PetGrid& g, const TofP
     const long long sa = sel3(g.stride, k.a), sb = sel3(g.stride, k.b), sc = sel3(g.stride, k.c);
     const int nb = sel3(g.n, k.b), nc = sel3(g.n, k.c);
     for (int i = k.i0; i <= k.i1; ++i) {
-        const float wt = kTof ? tof_weight(k, tp, cb, tof_tab, i) : 1.f;
+        const float wt = kTof ? tof_weight(k.l0, k.dl, tp, cb, tof_tab, i) : 1.f;
         const float u = fmaf((float)i, k.du, k.u0);
         const float w = fmaf((float)i, k.dw, k.w0);
         const float fu = floorf(u), fw = floorf(w);
@@ -383,33 +384,57 @@ __global__ void __launch_bounds__(kPetThreads) pet_lm_kernel(LmArgs a)
 // per voxel afterwards.  The lines of one axis go together (x, then y), so
 // that one axis's quads are in use at a time; lines along z, which a
 // cylindrical scanner hardly has, walk the image.
-// Bound by L1's rate of one line a cycle: a warp's 32 lanes touch 32 lines a
-// sample each way, about 1.7 cycles a sample for the gather and 2.0 for the
-// scatter.  Measured, image walk -> quads: 204 x 204 x 154 with time of
-// flight, 1 M events, 2.89 -> 2.09 ms; without, 3.27 -> 2.20 ms; 128 x 128 x
-// 90, 1 M lines, forward 1.17 -> 0.63 ms, back 1.36 -> 0.77 ms.  64 registers
-// (32 warps an SM) are worth more than a wider batch: 2.79 -> 2.20 ms.
-// Tried and not better: gathering and scattering in separate launches (2.71
-// ms), the time-of-flight lines slab by slab along the axis (2.27 ms).
+// Bound by L1's rate of one line a cycle.  With a line of response to a lane
+// and cells in plane order, a warp's 32 lanes touched 32 lines a sample each
+// way (1.7 cycles a sample for the gather, 2.0 for the scatter).  Four lanes
+// now walk a line together, on consecutive planes, and the cells lie in
+// 128-byte bricks of 4 planes x 2 u x 1 w, so that the four share about two
+// lines (along the axis a line moves by half a cell in u and less in w).
+// Measured, image walk -> quads in plane order -> bricks: an iteration of 3 M
+// events in 3 subsets at 204 x 204 x 154 with time of flight 9.7 -> 6.95 ->
+// 5.58 ms; 128 x 128 x 90, 1 M lines without, forward and back 2.60 -> 1.46 ->
+// 1.23 ms.  64 registers (32 warps an SM) are worth more than a wider batch:
+// 2.79 -> 2.20 ms a subset.  Tried and not better: gathering and scattering in
+// separate launches (2.71 ms), the time-of-flight lines slab by slab along the
+// axis (2.27 ms).
 
 constexpr int kQuadThreads = 128;
 
-// Cells of axis AX's lattice: planes of (nb + 1) x (nz + 1).
+// Where cell (u, w) of plane q lies in axis AX's lattice of na planes of
+// (nb + 1) x (nz + 1) cells: bricks of 4 planes x 2 u, 128 bytes, side by side
+// along w, the planes of one u next to each other in a brick.
+struct QuadLattice {
+    int w, u2, na4;  // cells along w, bricks along u and along the axis
+};
+
+__host__ __device__ inline QuadLattice quad_lattice(const PetGrid& g, int ax)
+{
+    return {g.n[2] + 1, (g.n[1 - ax] + 2) >> 1, (g.n[ax] + 3) >> 2};
+}
+
+__device__ __forceinline__ int quad_at(const QuadLattice& l, int q, int u, int w)
+{
+    return ((((q >> 2) * l.u2 + (u >> 1)) * l.w + w) << 3) + ((u & 1) << 2) + (q & 3);
+}
+
 __host__ __device__ inline long long quad_cells(const PetGrid& g, int ax)
 {
-    return (long long)g.n[ax] * (g.n[1 - ax] + 1) * (g.n[2] + 1);
+    const QuadLattice l = quad_lattice(g, ax);
+    return 8ll * l.na4 * l.u2 * l.w;
 }
 
 template <int AX>
 __global__ void __launch_bounds__(kPetThreads) pet_quads_kernel(const float* __restrict__ img, float4* __restrict__ quads,
                                                                 PetGrid g)
 {
-    const int nb = g.n[1 - AX], nc = g.n[2];
+    const int na = g.n[AX], nb = g.n[1 - AX], nc = g.n[2];
     const int sb = AX == 0 ? nc : g.n[1] * nc, sa = AX == 0 ? g.n[1] * nc : nc;  // voxels < 2^31 (use_quads)
+    const QuadLattice l = quad_lattice(g, AX);
     const int total = (int)quad_cells(g, AX);
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
-        const int w = c % (nc + 1), r = c / (nc + 1);
-        const int u = r % (nb + 1), q = r / (nb + 1);
+        const int k = c >> 3, w = k % l.w, r = k / l.w;
+        const int u = (r % l.u2) * 2 + ((c >> 2) & 1), q = (r / l.u2) * 4 + (c & 3);
+        if (q >= na || u > nb) continue;  // a brick's cells past the lattice: never read
         const float* p = img + (long long)q * sa + (long long)(u - 1) * sb + (w - 1);
         const bool u0 = u > 0, u1 = u < nb, w0 = w > 0, w1 = w < nc;
         quads[c] = make_float4(u0 && w0 ? __ldg(p) : 0.f, u0 && w1 ? __ldg(p + 1) : 0.f, u1 && w0 ? __ldg(p + sb) : 0.f,
@@ -417,53 +442,69 @@ __global__ void __launch_bounds__(kPetThreads) pet_quads_kernel(const float* __r
     }
 }
 
-// bp += the accumulated quads of axis AX.
+// bp += the accumulated quads of axis AX.  Threads walk voxels in the order of
+// the bricks (4 planes x 2 along b, then z), so that a warp's reads share lines.
 template <int AX>
 __global__ void __launch_bounds__(kPetThreads) pet_fold_kernel(const float4* __restrict__ quads, float* __restrict__ bp,
                                                                PetGrid g)
 {
-    const int nb = g.n[1 - AX], nc = g.n[2];
-    const int total = g.n[0] * g.n[1] * nc;
+    const int na = g.n[AX], nb = g.n[1 - AX], nc = g.n[2];
+    const int sb = AX == 0 ? nc : g.n[1] * nc, sa = AX == 0 ? g.n[1] * nc : nc;
+    const QuadLattice l = quad_lattice(g, AX);
+    const int b2 = (nb + 1) >> 1, total = 8 * l.na4 * b2 * nc;  // at most quad_cells
     const float* q1 = reinterpret_cast<const float*>(quads);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int z = i % nc, r = i / nc;
-        const int y = r % g.n[1], x = r / g.n[1];
-        const int q = AX == 0 ? x : y, b = AX == 0 ? y : x;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
+        const int k = c >> 3, z = k % nc, r = k / nc;
+        const int b = (r % b2) * 2 + ((c >> 2) & 1), q = (r / b2) * 4 + (c & 3);
+        if (q >= na || b >= nb) continue;
         // cell (u, w) of the lattice is lattice point (u - 1, w - 1)
-        const long long lo = ((long long)q * (nb + 1) + b) * (nc + 1) + z, hi = lo + nc + 1;
-        bp[i] += (__ldg(q1 + 4 * (hi + 1)) + __ldg(q1 + 4 * hi + 1)) + (__ldg(q1 + 4 * (lo + 1) + 2) + __ldg(q1 + 4 * lo + 3));
+        const long long lo = quad_at(l, q, b, z), hi = quad_at(l, q, b + 1, z);  // w + 1 is 8 cells on
+        bp[q * sa + b * sb + z] += (__ldg(q1 + 4 * (hi + 8)) + __ldg(q1 + 4 * hi + 1)) +
+                                   (__ldg(q1 + 4 * (lo + 8) + 2) + __ldg(q1 + 4 * lo + 3));
     }
 }
 
-// One batch of kBatch samples of a line over axis AX's quads: the cell of
-// each (-1 outside the image), its in-cell fractions and its weight.
-constexpr int kBatch = 4;
+// A line as the four lanes that walk it together see it: Walk's fields, and
+// val, what a back projection spreads (kModeBack) or the line's multiplier
+// (kModeEm).  i1 < i0: nothing to visit.
+struct QuadLine {
+    int q0, i0, i1;
+    float u0, w0, du, dw, step, l0, dl, cb, val;
+};
+
+// One batch of kBatch samples of a lane, four planes apart, from sample i on:
+// the cell of each (-1 outside the image or the line), its in-cell fractions
+// and its weight.
+constexpr int kBatch = 4, kQuadLanes = 4;
 struct QuadBatch {
     int cell[kBatch];
     float tu[kBatch], tw[kBatch], wt[kBatch];
 };
 
 template <bool kTof>
-__device__ __forceinline__ void quad_batch(QuadBatch& s, const Walk& k, int i, int nb, int nc, const TofParams& tp,
-                                           float cb, const float* tof_tab)
+__device__ __forceinline__ void quad_batch(QuadBatch& s, const QuadLine& k, int i, int nb, int nc, const QuadLattice& l,
+                                           const TofParams& tp, const float* tof_tab)
 {
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
-        const float f = (float)(i + j);
+        const int ij = i + j * kQuadLanes;
+        const float f = (float)ij;
         const float u = fmaf(f, k.du, k.u0), w = fmaf(f, k.dw, k.w0);
         const float fu = floorf(u), fw = floorf(w);
-        const bool in = i + j <= k.i1 && fu >= -1.f && fu <= (float)(nb - 1) && fw >= -1.f && fw <= (float)(nc - 1);
-        s.cell[j] = in ? ((k.q0 + i + j) * (nb + 1) + (int)fu + 1) * (nc + 1) + (int)fw + 1 : -1;
+        const bool in = ij >= k.i0 && ij <= k.i1 && fu >= -1.f && fu <= (float)(nb - 1) && fw >= -1.f &&
+                        fw <= (float)(nc - 1);
+        s.cell[j] = in ? quad_at(l, k.q0 + ij, (int)fu + 1, (int)fw + 1) : -1;
         s.tu[j] = u - fu;
         s.tw[j] = w - fw;
-        s.wt[j] = kTof ? tof_weight(k, tp, cb, tof_tab, i + j) : 1.f;
+        s.wt[j] = kTof ? tof_weight(k.l0, k.dl, tp, k.cb, tof_tab, ij) : 1.f;
     }
 }
 
 // The walk of pet_lm_kernel over quads, for the lines of principal axis AX.
 // A CTA collects the axis's lines from its share of the events in a queue in
 // shared memory and walks them a CTA at a time, so that its threads stay busy
-// whatever the mix of axes.
+// whatever the mix of axes.  Each thread prepares one line; four lanes then
+// walk a line together, eight lines of the warp at a time.
 template <int kMode, bool kTof, int AX>
 __global__ void __launch_bounds__(kQuadThreads, 8) pet_quad_kernel(LmArgs a)
 {
@@ -474,7 +515,8 @@ __global__ void __launch_bounds__(kQuadThreads, 8) pet_quad_kernel(LmArgs a)
         for (int i = threadIdx.x; i <= kTofTab; i += blockDim.x) tof_s[i] = __ldg(a.tof_tab + i);
     if (threadIdx.x == 0) queued = 0;
     __syncthreads();
-    const int nb = a.g.n[1 - AX], nc = a.g.n[2], lane = threadIdx.x & 31;
+    const int nb = a.g.n[1 - AX], nc = a.g.n[2], lane = threadIdx.x & 31, sub = lane & (kQuadLanes - 1);
+    const QuadLattice lat = quad_lattice(a.g, AX);
     double cons = 0.0, used = 0.0;
     long long next = blockIdx.x * (long long)kQuadThreads;
     int have = 0;  // lines in the queue (the same in every thread)
@@ -502,33 +544,80 @@ __global__ void __launch_bounds__(kQuadThreads, 8) pet_quad_kernel(LmArgs a)
         __syncthreads();  // taken; the queue may be filled again
         if (threadIdx.x == 0) queued = have;
         __syncthreads();
-        if (t < 0) continue;
-        const long long e = a.first + t * a.stride;
-        Walk k;
-        float cb = 0.f;
-        const bool hit = walk_setup<kTof>(a.lors + 6 * e, a.g, k, a.tof, kTof ? __ldg(a.tof_bin + e) : 0, cb);
-        auto scatter = [&](float sv) {
-            for (int i = k.i0; i <= k.i1; i += kBatch) {
-                QuadBatch s;
-                quad_batch<kTof>(s, k, i, nb, nc, a.tof, cb, tof_s);
-#pragma unroll
-                for (int j = 0; j < kBatch; ++j) {
-                    if (s.cell[j] < 0) continue;
-                    const float v = sv * s.wt[j], v0 = v * (1.f - s.tu[j]), v1 = v * s.tu[j], w0 = 1.f - s.tw[j];
-                    atomicAdd(a.bquads + s.cell[j], make_float4(v0 * w0, v0 * s.tw[j], v1 * w0, v1 * s.tw[j]));
+        // this thread's line
+        const long long e = t < 0 ? -1 : a.first + t * a.stride;
+        QuadLine own{};
+        own.i1 = -1;
+        float add = 0.f;  // kModeEm: the additive term
+        if (t >= 0) {
+            Walk k;
+            float cb = 0.f;
+            const bool hit = walk_setup<kTof>(a.lors + 6 * e, a.g, k, a.tof, kTof ? __ldg(a.tof_bin + e) : 0, cb);
+            if (kMode == kModeBack) own.val = __ldg(a.vals + e) * (a.mult ? __ldg(a.mult + e) : 1.f);
+            if (kMode == kModeFwd) own.val = a.mult ? __ldg(a.mult + e) : 1.f;
+            if (kMode == kModeEm) {
+                own.val = __ldg(a.mult + e);
+                add = a.s ? __ldg(a.s + e) : 0.f;
+            }
+            if (hit && !(kMode == kModeBack && own.val == 0.f)) {
+                own.q0 = k.q0;
+                own.i0 = k.i0;
+                own.i1 = k.i1;
+                own.u0 = k.u0;
+                own.w0 = k.w0;
+                own.du = k.du;
+                own.dw = k.dw;
+                own.step = k.step;
+                if (kTof) {
+                    own.l0 = k.l0;
+                    own.dl = k.dl;
+                    own.cb = cb;
                 }
             }
-        };
-        if (kMode == kModeBack) {
-            const float val = __ldg(a.vals + e) * (a.mult ? __ldg(a.mult + e) : 1.f);
-            if (hit && val != 0.f) scatter(val * k.step);
-            continue;
         }
-        float acc = 0.f;
-        if (hit) {
-            for (int i = k.i0; i <= k.i1; i += kBatch) {
+#pragma unroll 1
+        for (int p = 0; p < kQuadLanes; ++p) {
+            const int src = p * (32 / kQuadLanes) + lane / kQuadLanes;
+            auto from = [&](auto v) { return __shfl_sync(0xffffffffu, v, src); };
+            const long long el = from(e);
+            QuadLine k{};
+            k.q0 = from(own.q0);
+            k.i0 = from(own.i0);
+            k.i1 = from(own.i1);
+            k.u0 = from(own.u0);
+            k.w0 = from(own.w0);
+            k.du = from(own.du);
+            k.dw = from(own.dw);
+            k.step = from(own.step);
+            k.val = from(own.val);
+            if (kTof) {
+                k.l0 = from(own.l0);
+                k.dl = from(own.dl);
+                k.cb = from(own.cb);
+            }
+            // lane `sub` takes the planes q with q % 4 == sub: the four lanes'
+            // samples of a step share a brick unless the line leaves it
+            const int first = k.i0 - ((k.q0 + k.i0) & (kQuadLanes - 1)) + sub;
+            auto scatter = [&](float sv) {
+                for (int i = first; i <= k.i1; i += kBatch * kQuadLanes) {
+                    QuadBatch s;
+                    quad_batch<kTof>(s, k, i, nb, nc, lat, a.tof, tof_s);
+#pragma unroll
+                    for (int j = 0; j < kBatch; ++j) {
+                        if (s.cell[j] < 0) continue;
+                        const float v = sv * s.wt[j], v0 = v * (1.f - s.tu[j]), v1 = v * s.tu[j], w0 = 1.f - s.tw[j];
+                        atomicAdd(a.bquads + s.cell[j], make_float4(v0 * w0, v0 * s.tw[j], v1 * w0, v1 * s.tw[j]));
+                    }
+                }
+            };
+            if (kMode == kModeBack) {
+                scatter(k.val * k.step);
+                continue;
+            }
+            float acc = 0.f;
+            for (int i = first; i <= k.i1; i += kBatch * kQuadLanes) {
                 QuadBatch s;
-                quad_batch<kTof>(s, k, i, nb, nc, a.tof, cb, tof_s);
+                quad_batch<kTof>(s, k, i, nb, nc, lat, a.tof, tof_s);
                 float4 v[kBatch];
 #pragma unroll
                 for (int j = 0; j < kBatch; ++j)
@@ -541,18 +630,22 @@ __global__ void __launch_bounds__(kQuadThreads, 8) pet_quad_kernel(LmArgs a)
                     acc = fmaf(s.wt[j], fmaf(s.tu[j], hi, (1.f - s.tu[j]) * lo), acc);
                 }
             }
-        }
-        const float line = hit ? acc * k.step : 0.f;
-        if (kMode == kModeFwd) {
-            a.out[e] = a.mult ? __ldg(a.mult + e) * line : line;
-        } else {  // kModeEm
-            const float m = __ldg(a.mult + e);
-            const float p = m * line;
-            const float den = p + (a.s ? __ldg(a.s + e) : 0.f);
-            if (!(den > 0.f)) continue;
-            cons += (double)p / (double)den;
-            used += 1.0;
-            if (hit) scatter(m / den * k.step);
+#pragma unroll
+            for (int o = 1; o < kQuadLanes; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            const float line = acc * k.step;  // 0 for a line that misses (step 0)
+            if (kMode == kModeFwd) {
+                if (el >= 0 && sub == 0) a.out[el] = a.mult ? k.val * line : line;
+            } else {  // kModeEm
+                const float pr = k.val * line;
+                const float den = pr + from(add);
+                if (el >= 0 && den > 0.f) {
+                    if (sub == 0) {
+                        cons += (double)pr / (double)den;
+                        used += 1.0;
+                    }
+                    scatter(k.val / den * k.step);
+                }
+            }
         }
     }
     if (kMode == kModeEm && a.diag) block_add2(cons, used, a.diag);
@@ -789,7 +882,7 @@ LmArgs base_args(const pet_plan* p, const float* lors, long long n)
 bool use_quads(pet_plan* p, long long lines, cudaStream_t st)
 {
     const long long cells = std::max(quad_cells(p->grid, 0), quad_cells(p->grid, 1));
-    if (lines < p->voxels / 32 || cells >= (1ll << 31) || p->voxels >= (1ll << 31) || p->quads_failed) return false;
+    if (lines < p->voxels / 32 || cells >= (1ll << 31) - (1ll << 23) || p->voxels >= (1ll << 31) || p->quads_failed) return false;
     if (p->quads && p->bquads) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
