@@ -94,4 +94,11 @@ __device__ __forceinline__ void prefetch_line_l2(const void* p)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory");
 }
 
+// See launch_early (internal.h).  wait_prerequisites returns once the kernels
+// before this one in the stream have completed and their writes are visible;
+// without them, or in an ordinary launch, at once.  What follows reads their
+// output with plain loads: a read-only one (__ldg) may be moved before it.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 }  // namespace spect

@@ -147,37 +147,12 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) blur_back_kernel(BlurBackArg
     const float* aplane = a.atten ? a.atten + (size_t)angle * n * n * nz : nullptr;
     const int rp = t.npad >> 1;
 
-    // The projection window of this angle (all ones without a projection),
-    // times the angle's T_fov weights when the plan has them, zero outside
-    // the detector.
-    const float* pr = a.proj ? a.proj + (size_t)b * a.proj_bstride + (size_t)sidx * n * nz : nullptr;
-    const float* fv = a.fov ? a.fov + (size_t)angle * n * nz : nullptr;
-    {
-        const int wq = (t.ktpad >> 1) + t.rh;  // column pairs of the window
-#pragma unroll 4
-        for (int it = tid; it < rp * wq; it += blockDim.x) {
-            const int jp = it / wq, cq = it - jp * wq;
-            const int k = kw0 + 2 * cq;
-            float2 v[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = 2 * jp + h;
-                v[h] = make_float2(0.f, 0.f);
-                if (j < n && k >= klo && k < khi) {
-                    v[h] = pr ? __ldg(reinterpret_cast<const float2*>(pr + (size_t)j * nz + k)) : make_float2(1.f, 1.f);
-                    if (fv) {
-                        const float2 m = __ldg(reinterpret_cast<const float2*>(fv + (size_t)j * nz + k));
-                        v[h] = make_float2(v[h].x * m.x, v[h].y * m.y);
-                    }
-                }
-            }
-            P[jp * t.sp + cq] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
-        }
-        // the j-blur's zero rows above and below the plane
-        for (int it = tid; it < t.pad_rows * kSq; it += blockDim.x) {
-            Q[it - t.pad_rows * kSq] = make_float4(0.f, 0.f, 0.f, 0.f);
-            Q[it + rp * kSq] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+    launch_dependents();
+
+    // the j-blur's zero rows above and below the plane
+    for (int it = tid; it < t.pad_rows * kSq; it += blockDim.x) {
+        Q[it - t.pad_rows * kSq] = make_float4(0.f, 0.f, 0.f, 0.f);
+        Q[it + rp * kSq] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     int i_lo, i_hi;
     chunk_planes(bounds_g, work_g, n, a.chunks, chunk, i_lo, i_hi);
@@ -186,15 +161,42 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) blur_back_kernel(BlurBackArg
         tp.load(taps_g, i_lo);
         tp.store(taps_s, i_lo);
     }
+    // a buffered plane is whole (one tile): one copy
+    const uint32_t a_bytes = 4u * (uint32_t)(n * nz);
     if (kSmemA && tid == 0) {
         mbar_init(bar, 1);
         mbar_init_fence();
+        if (i_lo < i_hi) tma_load_1d(smem_u32(As), aplane + (size_t)i_lo * n * nz, a_bytes, bar);
     }
-    if (aplane && i_lo < i_hi) prefetch_plane_l2(aplane + (size_t)i_lo * n * nz, n, nz, kt0, kt0 + KT);
+    if (!kSmemA && aplane && i_lo < i_hi) prefetch_plane_l2(aplane + (size_t)i_lo * n * nz, n, nz, kt0, kt0 + KT);
+    wait_prerequisites();  // up to here plan data only
+
+    // The projection window of this angle (all ones without a projection),
+    // times the angle's T_fov weights when the plan has them, zero outside
+    // the detector.
+    const float* pr = a.proj ? a.proj + (size_t)b * a.proj_bstride + (size_t)sidx * n * nz : nullptr;
+    const float* fv = a.fov ? a.fov + (size_t)angle * n * nz : nullptr;
+    const int wq = (t.ktpad >> 1) + t.rh;  // column pairs of the window
+#pragma unroll 4
+    for (int it = tid; it < rp * wq; it += blockDim.x) {
+        const int jp = it / wq, cq = it - jp * wq;
+        const int k = kw0 + 2 * cq;
+        float2 v[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = 2 * jp + h;
+            v[h] = make_float2(0.f, 0.f);
+            if (j < n && k >= klo && k < khi) {
+                v[h] = pr ? *reinterpret_cast<const float2*>(pr + (size_t)j * nz + k) : make_float2(1.f, 1.f);
+                if (fv) {
+                    const float2 m = __ldg(reinterpret_cast<const float2*>(fv + (size_t)j * nz + k));
+                    v[h] = make_float2(v[h].x * m.x, v[h].y * m.y);
+                }
+            }
+        }
+        P[jp * t.sp + cq] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
+    }
     __syncthreads();
-    // a buffered plane is whole (one tile): one copy
-    const uint32_t a_bytes = 4u * (uint32_t)(n * nz);
-    if (kSmemA && tid == 0 && i_lo < i_hi) tma_load_1d(smem_u32(As), aplane + (size_t)i_lo * n * nz, a_bytes, bar);
     float* bvol = a.bvol + item * (size_t)n * n * nz;
     // this thread's first z-blur strip (row pair, strip) and j-blur strip
     // (column pair, strip)
@@ -246,9 +248,8 @@ cudaError_t launch_sq(const BlurBackArgs& a, cudaStream_t st)
 {
     cudaError_t e = allow_big_smem(blur_back_kernel<kSq, kSmemA, kHigh>, g_blur_back_smem_mask<kSq, kSmemA, kHigh>);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.chunks * a.t.ntiles, a.n_sel, a.batch);
-    blur_back_kernel<kSq, kSmemA, kHigh><<<grid, a.t.threads, a.t.smem, st>>>(a);
-    return cudaGetLastError();
+    const dim3 grid(a.chunks * a.t.ntiles, a.n_sel, a.batch);
+    return launch_early(blur_back_kernel<kSq, kSmemA, kHigh>, a, grid, a.t.threads, a.t.smem, st);
 }
 
 template <int kSq, bool kSmemA, bool kHigh>

@@ -10,6 +10,7 @@
 // holds at most 4 + 8/2 + 1 = 9 lattice points, hence kMaxCand = 9.
 #include <cuda_runtime.h>
 
+#include "async_copy.cuh"
 #include "geometry.cuh"
 #include "internal.h"
 #include "update.cuh"
@@ -63,6 +64,8 @@ cudaError_t launch_gather_tables(const float4* cs, int n, int nz, int n_angles, 
 // angle's entries in table order, so it is deterministic.
 __global__ void __launch_bounds__(256) gather_kernel(GatherArgs a)
 {
+    launch_dependents();
+    wait_prerequisites();
     const int n = a.n, nz = a.nz, zw = nz >> 2;
     const int lane = threadIdx.x & 31;
     const long gw = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -97,8 +100,8 @@ __global__ void __launch_bounds__(256) gather_kernel(GatherArgs a)
         const float* b1 = bb + (size_t)(g + 1) * vol;
 #pragma unroll
         for (int e = 0; e < kMaxCand; ++e) {
-            v0[e] = e0[e].y != 0 ? __ldg(reinterpret_cast<const float4*>(b0 + e0[e].x)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            v1[e] = e1[e].y != 0 ? __ldg(reinterpret_cast<const float4*>(b1 + e1[e].x)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v0[e] = e0[e].y != 0 ? *reinterpret_cast<const float4*>(b0 + e0[e].x) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v1[e] = e1[e].y != 0 ? *reinterpret_cast<const float4*>(b1 + e1[e].x) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int e = 0; e < kMaxCand; ++e) {
@@ -145,9 +148,7 @@ cudaError_t launch_gather(const GatherArgs& a, cudaStream_t st)
     else
         warps = ((long)a.n * a.n + (32 / a.lanes_per_col) - 1) / (32 / a.lanes_per_col);
     const long blocks = (warps * 32 + 255) / 256;
-    dim3 grid((unsigned)blocks, a.batch);
-    gather_kernel<<<grid, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_early(gather_kernel, a, dim3((unsigned)blocks, a.batch), 256, 0, st);
 }
 
 }  // namespace spect

@@ -283,6 +283,7 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
     const float* bvol_b = a.bvol + (size_t)b * a.n_sel * vol;
     const size_t tab_stride = (size_t)a.n_tiles * (kGtSliceBytes / 8);  // int2 per angle
 
+    launch_dependents();
     if (threadIdx.x == 0) {
         for (int q = 0; q <= S; ++q) mbar_init(smem_u32(bars + q), 1);
         mbar_init_fence();
@@ -310,6 +311,9 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
         }
         desc_ok = mbar_wait(dbar, 0);
         __syncwarp();
+    }
+    wait_prerequisites();  // up to here plan data only
+    if (producer) {
         if (desc_ok)
             for (int g = 0; g < S - 1 && g < a.n_sel; ++g) issue(g);
     }
@@ -396,7 +400,7 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
             i4[u] = ((((size_t)x * a.n + y) * a.nz + z0) >> 2) + lane;  // float4 of the volume
             xv[u] = sv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (live[u] && need_x) xv[u] = out_b[i4[u]];
-            if (live[u] && upd) sv[u] = __ldg(reinterpret_cast<const float4*>(a.upd.sens) + i4[u]);
+            if (live[u] && upd) sv[u] = reinterpret_cast<const float4*>(a.upd.sens)[i4[u]];
         }
 #pragma unroll
         for (int u = 0; u < kEpi; ++u) {
@@ -435,9 +439,9 @@ cudaError_t launch_gather_tiled_t(const GatherTiledArgs& a, cudaStream_t st)
         mask |= 1ull << (dev & 63);
     }
     if (a.n_sel > 32) return cudaErrorInvalidValue;  // warp 0 holds one angle id per lane
-    dim3 grid(a.n_tiles, a.batch, a.nz / a.zs);
-    gather_tiled_kernel<T><<<grid, kGatherTiledThreads, gather_tiled_smem(a.rows_cap, a.zs, T, a.stages, a.n_sel), st>>>(a);
-    return cudaGetLastError();
+    const dim3 grid(a.n_tiles, a.batch, a.nz / a.zs);
+    return launch_early(gather_tiled_kernel<T>, a, grid, kGatherTiledThreads,
+                        gather_tiled_smem(a.rows_cap, a.zs, T, a.stages, a.n_sel), st);
 }
 
 cudaError_t launch_gather_tiled(const GatherTiledArgs& a, cudaStream_t st)

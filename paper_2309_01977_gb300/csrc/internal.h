@@ -46,6 +46,7 @@ struct PlaneTiling {
     int sq;       // Q stride between column pairs, in quads (odd): >= (npad + 2*rh) / 2
     int threads;  // CTA size (multiple of 32, <= kFwdThreads)
     int ipt;      // j-blur strips per thread (1..kMaxIpt)
+    int ctas;     // CTAs an SM holds (1 or 2)
     bool high;    // radii past kLowR, or several strips per thread: the kernel with every radius
     // Attenuation planes staged in shared memory by one bulk copy each, a
     // plane ahead (else A is read from global memory); byte offsets of the tap
@@ -57,6 +58,39 @@ struct PlaneTiling {
 
 // Shape of one back blur launch (blur_back.cuh).
 constexpr int kBackStrides[] = {9, 17, 33, 49, 65};  // strides of Q: half a tile's columns, rounded up to odd
+
+// Launch of a kernel that calls launch_dependents() at its start and
+// wait_prerequisites() (async_copy.cuh) before it touches what earlier
+// kernels of the stream write or read: its CTAs may take their SMs while the
+// last CTAs of the kernel before it still run, so that the launch and the part
+// of the kernel that needs only plan data (tables, barriers, shared-memory
+// zeros, the first attenuation plane) overlap that kernel's tail.  After any
+// other kernel or copy it starts as an ordinary launch does.  Measured, OSEM
+// with ordinary and with early launches: 64^3, 16 subiterations of 8 angles
+// 741 -> 654 us (BF16, 8 subiterations 467 -> 390); 96^3 x 12 x 8 968 -> 907;
+// 128^3 x 15 x 8 1766 -> 1717 (BF16 1430 -> 1400).
+// ctas > 0: with the smallest shared-memory carve-out that holds so many CTAs
+// (and the 1 KB that each takes on top); the rest of the SM's 256 KB is L1.
+constexpr size_t kSmSmem = 228 * 1024;
+template <class A>
+inline cudaError_t launch_early(void (*fn)(A), const A& args, dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                int ctas = 0)
+{
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    const size_t percent = ((smem + 1024) * ctas * 100 + kSmSmem - 1) / kSmSmem;  // rounded up
+    at[1].val.sharedMemCarveout = (unsigned)(percent < 100 ? percent : 100);
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = at;
+    c.numAttrs = ctas > 0 ? 2 : 1;
+    return cudaLaunchKernelEx(&c, fn, args);
+}
 
 // threads % width and threads / width of a grid of items, `width` to a row.
 struct ItemStep {

@@ -173,10 +173,12 @@ cudaError_t launch_diag_finalize(const double* part, int n_part, double* out3, c
 template <bool kDiag>
 __global__ void __launch_bounds__(256) forward_reduce_kernel(ReduceArgs a)
 {
+    launch_dependents();
+    wait_prerequisites();
     __shared__ double red[32];
     const int plane4 = a.plane >> 2;
     const size_t total4 = (size_t)a.items * plane4;
-    const float s = a.s_ptr ? __ldg(a.s_ptr) : a.s;
+    const float s = a.s_ptr ? *a.s_ptr : a.s;
     double d0 = 0.0, d1 = 0.0, d2 = 0.0;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total4; e += (size_t)gridDim.x * blockDim.x) {
         const int item = (int)(e / plane4);
@@ -210,7 +212,7 @@ __global__ void __launch_bounds__(256) forward_reduce_kernel(ReduceArgs a)
         float4 o = p;
         if (a.y) {
             const int angle = a.sel[item % a.n_sel];
-            const float4 yv = __ldg(reinterpret_cast<const float4*>(a.y) + (size_t)angle * plane4 + off4);
+            const float4 yv = reinterpret_cast<const float4*>(a.y)[(size_t)angle * plane4 + off4];
             const float pv[4] = {p.x, p.y, p.z, p.w};
             const float yy[4] = {yv.x, yv.y, yv.z, yv.w};
             float rv[4];
@@ -242,11 +244,8 @@ __global__ void __launch_bounds__(256) forward_reduce_kernel(ReduceArgs a)
 
 cudaError_t launch_forward_reduce(const ReduceArgs& a, int blocks, cudaStream_t st)
 {
-    if (a.diag_blocks)
-        forward_reduce_kernel<true><<<blocks, 256, 0, st>>>(a);
-    else
-        forward_reduce_kernel<false><<<blocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_early(a.diag_blocks ? forward_reduce_kernel<true> : forward_reduce_kernel<false>, a, dim3(blocks), 256, 0,
+                        st);
 }
 
 // Poisson log-likelihood (Table 1): sum_b y_b log(p_b + s) - (p_b + s), in

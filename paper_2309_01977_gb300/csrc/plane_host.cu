@@ -11,8 +11,6 @@ namespace {
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-constexpr size_t kSmSmem = 228 * 1024;  // shared memory of an SM; each resident CTA takes 1 KB on top of its own
-
 // Forward z tile of ktile columns; smem 0 where its strips do not fit.
 PlaneTiling make_tiling(int n, int nz, int rmax, int ktile, size_t cap, size_t limit)
 {
@@ -49,6 +47,7 @@ PlaneTiling make_tiling(int n, int nz, int rmax, int ktile, size_t cap, size_t l
     const int items = (t.ktpad / 2) * (t.npad / kStrip);
     const bool two = 2 * (t.smem + 1024) <= kSmSmem;
     t.threads = two && items <= kPlaneThreads / 2 ? kPlaneThreads / 2 : kPlaneThreads;
+    t.ctas = two && t.threads <= kPlaneThreads / 2 ? 2 : 1;
     t.ipt = (items + t.threads - 1) / t.threads;
     t.high = rmax > kLowR || t.ipt > 1;
     if (t.ipt > kMaxIpt || (size_t)t.off_taps + 2 * kTapRow * sizeof(float) > cap) t.smem = 0;

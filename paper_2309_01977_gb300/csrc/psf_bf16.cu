@@ -452,7 +452,7 @@ __device__ __forceinline__ void stage_rows(uint32_t b1, uint32_t b1_lo, TcTapRow
                 const int j = jr[r] < n ? jr[r] : wi;  // rows past n repeat a valid row; not stored
                 t[r] = rows[j];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) f[r][q] = __ldg(reinterpret_cast<const float4*>(xb + t[r].off[q] + k));
+                for (int q = 0; q < 4; ++q) f[r][q] = *reinterpret_cast<const float4*>(xb + t[r].off[q] + k);
                 av[r] = arow ? __ldg(reinterpret_cast<const float4*>(arow + (size_t)j * nz + k))
                              : make_float4(1.f, 1.f, 1.f, 1.f);
             }
@@ -482,7 +482,7 @@ __device__ __forceinline__ void stage_proj_rows(uint32_t b1, uint32_t b1_lo, con
     for (int j = wi; j < n; j += kWorkers) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (k < nz) {
-            v = pr ? __ldg(reinterpret_cast<const float4*>(pr + (size_t)j * nz + k)) : make_float4(1.f, 1.f, 1.f, 1.f);
+            v = pr ? *reinterpret_cast<const float4*>(pr + (size_t)j * nz + k) : make_float4(1.f, 1.f, 1.f, 1.f);
             if (fv) {
                 const float4 m = __ldg(reinterpret_cast<const float4*>(fv + (size_t)j * nz + k));
                 v = make_float4(v.x * m.x, v.y * m.y, v.z * m.z, v.w * m.w);
@@ -530,6 +530,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) forward_bf16_kernel(ForwardBf16
         mbar_init_fence();
     }
     const uint32_t tmem = tc_alloc(bars + kTmemSlot, a.tmem_cols);  // D1, D2, A2 (hi, lo)
+    launch_dependents();  // holding its tensor memory: a later kernel that waits for this one cannot keep it from it
     const uint32_t d1 = tmem, d2 = tmem + (uint32_t)n;
     const uint32_t a2hi = tmem + a2_tmem_col(n, 2), a2lo = a2hi + 64u;
     const uint32_t idesc = idesc_bf16(kTcM, n);
@@ -547,6 +548,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) forward_bf16_kernel(ForwardBf16
         return a.atten ? a.atten + ((size_t)angle * n + plane(p)) * n * nz : nullptr;
     };
 
+    // the issuing warp only reads plan data (the Toeplitz tiles)
+    if (np == 0 || warp != 0) wait_prerequisites();
     if (np == 0) {
         // a chunk without planes (more chunks than planes): its sum is zero
         for (int e = tid; e < n * nz; e += blockDim.x) dst[e] = 0.f;
@@ -657,6 +660,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) blur_back_bf16_kernel(BlurBackB
         mbar_init_fence();
     }
     const uint32_t tmem = tc_alloc(bars + kTmemSlot, a.tmem_cols);  // D1, D2[0], D2[1], A2 (hi, lo)
+    launch_dependents();  // holding its tensor memory: a later kernel that waits for this one cannot keep it from it
     const uint32_t d1 = tmem;
     const uint32_t a2hi = tmem + a2_tmem_col(n, 3), a2lo = a2hi + 64u;
     const uint32_t t_lo = base + 2u * kTile, b1 = base + 3u * kTile;
@@ -676,6 +680,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) blur_back_bf16_kernel(BlurBackB
         return a.atten ? a.atten + ((size_t)angle * n + plane(p)) * n * nz : nullptr;
     };
 
+    // the issuing warp only reads plan data (the Toeplitz tiles)
+    if (warp != 0) wait_prerequisites();
     if (np > 0 && warp == 0) {
         if (lane == 0) {
             TileLoads tl;  // slots 0, 1: T_hi; slot 2: T_lo
@@ -838,18 +844,14 @@ cudaError_t launch_forward_bf16(const ForwardBf16Args& a, cudaStream_t st)
 {
     cudaError_t e = raise_smem(forward_bf16_kernel, fwd_smem(kTcM), g_fwd_bf16_mask);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.chunks, a.n_sel, a.batch);
-    forward_bf16_kernel<<<grid, kTcThreads, fwd_smem(a.n), st>>>(a);
-    return cudaGetLastError();
+    return launch_early(forward_bf16_kernel, a, dim3(a.chunks, a.n_sel, a.batch), kTcThreads, fwd_smem(a.n), st);
 }
 
 cudaError_t launch_blur_back_bf16(const BlurBackBf16Args& a, cudaStream_t st)
 {
     cudaError_t e = raise_smem(blur_back_bf16_kernel, back_smem(kTcM), g_back_bf16_mask);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.chunks, a.n_sel, a.batch);
-    blur_back_bf16_kernel<<<grid, kTcThreads, back_smem(a.n), st>>>(a);
-    return cudaGetLastError();
+    return launch_early(blur_back_bf16_kernel, a, dim3(a.chunks, a.n_sel, a.batch), kTcThreads, back_smem(a.n), st);
 }
 
 }  // namespace spect
