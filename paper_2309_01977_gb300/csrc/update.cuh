@@ -45,9 +45,4 @@ __device__ __forceinline__ float4 update4_sv(const UpdateSpec& u, float4 x, floa
                        update1(u, x.z, bp.z, sv.z, gv.z, sa.z), update1(u, x.w, bp.w, sv.w, gv.w, sa.w));
 }
 
-__device__ __forceinline__ float4 update4(const UpdateSpec& u, float4 x, float4 bp, size_t i4)
-{
-    return update4_sv(u, x, bp, reinterpret_cast<const float4*>(u.sens)[i4], i4);
-}
-
 }  // namespace spect
