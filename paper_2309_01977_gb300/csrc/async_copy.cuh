@@ -101,4 +101,25 @@ __device__ __forceinline__ void prefetch_line_l2(const void* p)
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Barrier over all threads of the CTA's cluster; shared-memory writes before it
+// are visible to the cluster after it.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// 16 bytes at this CTA's shared address `addr`, in the shared memory of the
+// cluster's CTA `rank`.
+__device__ __forceinline__ float4 ld_peer_f4(uint32_t addr, uint32_t rank)
+{
+    uint32_t peer;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(addr), "r"(rank));
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(peer)
+                 : "memory");
+    return v;
+}
+
 }  // namespace spect

@@ -257,12 +257,16 @@ __device__ __forceinline__ void fma4(float4& a4, float w, const float4& v)
 // long to issue as an angle's sums), so that they overlap the sums.  Two
 // CTAs per SM (their shared memory allows two; 18 warps cap the registers
 // at 96).
-template <int T>
+// kPair: the two CTAs of a cluster take half of the angles each, and the first
+// adds up both (launches of fewer CTAs than SMs, see gather_pair_fits).
+template <int T, bool kPair>
 __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(GatherTiledArgs a)
 {
     static_assert(T == kGtT, "strip tables are built for 8 x 8 tiles");
     extern __shared__ __align__(16) float4 gsm[];
-    const int tile = blockIdx.x, b = blockIdx.y;
+    const int tile = kPair ? blockIdx.x >> 1 : blockIdx.x, half = kPair ? blockIdx.x & 1 : 0, b = blockIdx.y;
+    const int per = kPair ? (a.n_sel + 1) >> 1 : a.n_sel, g0 = half * per;
+    const int n_sel = kPair ? min(per, a.n_sel - g0) : a.n_sel;
     const int tiles_x = (a.n + T - 1) / T;
     const int tx = tile % tiles_x, ty = tile / tiles_x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -279,8 +283,8 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
     float4* bufs = gsm;
     uint64_t* bars = reinterpret_cast<uint64_t*>(gsm + S * buf_f4);
     int* sdesc = reinterpret_cast<int*>(gsm + S * buf_f4 + (S + 2) / 2);
-    int* s_sel = sdesc + a.n_sel * kFpDescInts;
-    const float* bvol_b = a.bvol + (size_t)b * a.n_sel * vol;
+    int* s_sel = sdesc + n_sel * kFpDescInts;
+    const float* bvol_b = a.bvol + ((size_t)b * a.n_sel + g0) * vol;
     const size_t tab_stride = (size_t)a.n_tiles * (kGtSliceBytes / 8);  // int2 per angle
 
     launch_dependents();
@@ -301,10 +305,10 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
     bool desc_ok = true;
     if (producer) {
         const uint32_t dbar = smem_u32(bars + S);
-        if (lane == 0) mbar_expect_tx(dbar, (uint32_t)a.n_sel * kFpDescInts * 4u);
+        if (lane == 0) mbar_expect_tx(dbar, (uint32_t)n_sel * kFpDescInts * 4u);
         __syncwarp();
-        if (lane < a.n_sel) {
-            const int ag = __ldg(a.sel + lane);
+        if (lane < n_sel) {
+            const int ag = __ldg(a.sel + g0 + lane);
             s_sel[lane] = ag;
             bulk_load(smem_u32(sdesc + lane * kFpDescInts), a.desc + ((size_t)ag * a.n_tiles + tile) * kFpDescInts,
                       kFpDescInts * 4u, dbar);
@@ -315,7 +319,7 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
     wait_prerequisites();  // up to here plan data only
     if (producer) {
         if (desc_ok)
-            for (int g = 0; g < S - 1 && g < a.n_sel; ++g) issue(g);
+            for (int g = 0; g < S - 1 && g < n_sel; ++g) issue(g);
     }
 
     float4 acc[kCols];
@@ -323,10 +327,10 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
     for (int k = 0; k < kCols; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     bool ok = true;
     int g = 0;
-    for (; g < a.n_sel; ++g) {
+    for (; g < n_sel; ++g) {
         // buffer (g + S - 1) % S was last read by angle g - 1, before the
         // barrier that ended it
-        if (producer && desc_ok && g + S - 1 < a.n_sel) {
+        if (producer && desc_ok && g + S - 1 < n_sel) {
             fence_async_smem();
             issue(g + S - 1);
         }
@@ -374,9 +378,28 @@ __global__ void __launch_bounds__(kGatherTiledThreads, 2) gather_tiled_kernel(Ga
         // g .. g + S - 2) one more bounded wait before the CTA's shared memory
         // goes away
         if (threadIdx.x == 0) atomicExch(a.err, SPECT_ETIMEDOUT);
-        for (int h = g; h < g + S - 1 && h < a.n_sel; ++h) mbar_wait(smem_u32(bars + h % S), (uint32_t)((h / S) & 1));
-        return;
+        for (int h = g; h < g + S - 1 && h < n_sel; ++h) mbar_wait(smem_u32(bars + h % S), (uint32_t)((h / S) & 1));
     }
+    if (kPair) {
+        // the second CTA's sums go to the first through its shared memory
+        // (the footprint buffers, which no copy uses any more); both reach
+        // both barriers whatever happened before
+        const uint32_t at = smem_u32(bufs) + 16u * threadIdx.x;
+        constexpr uint32_t row = 16u * 32u * kGatherSumWarps;
+        if (half == 1 && !producer)
+#pragma unroll
+            for (int k = 0; k < kCols; ++k) bufs[threadIdx.x + k * 32 * kGatherSumWarps] = acc[k];
+        cluster_sync();
+        if (half == 0 && !producer)
+#pragma unroll
+            for (int k = 0; k < kCols; ++k) {
+                const float4 v = ld_peer_f4(at + k * row, 1);
+                acc[k] = make_float4(acc[k].x + v.x, acc[k].y + v.y, acc[k].z + v.z, acc[k].w + v.w);
+            }
+        cluster_sync();
+        if (half == 1) return;
+    }
+    if (!ok) return;
 
     // epilogue: store, accumulate, or the fused OSEM update.  The image
     // values and sensitivities of kEpi columns are loaded before any of their
@@ -423,7 +446,13 @@ size_t gather_tiled_smem(int rows_cap, int zs, int T, int stages, int n_sel)
     return bufs + bars + (size_t)n_sel * (kFpDescInts + 1) * sizeof(int);
 }
 
-template <int T>
+bool gather_pair_fits(int rows_cap, int zs, int stages)
+{
+    return stages * ((size_t)rows_cap * zs * sizeof(float) + (size_t)kGtSliceBytes) >=
+           sizeof(float4) * 32 * kGatherSumWarps * kGtT;
+}
+
+template <int T, bool kPair>
 cudaError_t launch_gather_tiled_t(const GatherTiledArgs& a, cudaStream_t st)
 {
     static unsigned long long mask = 0;
@@ -434,19 +463,20 @@ cudaError_t launch_gather_tiled_t(const GatherTiledArgs& a, cudaStream_t st)
         int optin = 0;
         e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(gather_tiled_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+        e = cudaFuncSetAttribute(gather_tiled_kernel<T, kPair>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
         if (e != cudaSuccess) return e;
         mask |= 1ull << (dev & 63);
     }
     if (a.n_sel > 32) return cudaErrorInvalidValue;  // warp 0 holds one angle id per lane
-    const dim3 grid(a.n_tiles, a.batch, a.nz / a.zs);
-    return launch_early(gather_tiled_kernel<T>, a, grid, kGatherTiledThreads,
-                        gather_tiled_smem(a.rows_cap, a.zs, T, a.stages, a.n_sel), st);
+    const dim3 grid(a.n_tiles * (kPair ? 2 : 1), a.batch, a.nz / a.zs);
+    return launch_early(gather_tiled_kernel<T, kPair>, a, grid, kGatherTiledThreads,
+                        gather_tiled_smem(a.rows_cap, a.zs, T, a.stages, a.n_sel), st, 0, kPair ? 2 : 1);
 }
 
 cudaError_t launch_gather_tiled(const GatherTiledArgs& a, cudaStream_t st)
 {
-    return a.T == kGtT ? launch_gather_tiled_t<kGtT>(a, st) : cudaErrorInvalidValue;
+    if (a.T != kGtT) return cudaErrorInvalidValue;
+    return a.pair ? launch_gather_tiled_t<kGtT, true>(a, st) : launch_gather_tiled_t<kGtT, false>(a, st);
 }
 
 }  // namespace spect

@@ -71,24 +71,33 @@ constexpr int kBackStrides[] = {9, 17, 33, 49, 65};  // strides of Q: half a til
 // 128^3 x 15 x 8 1766 -> 1717 (BF16 1430 -> 1400).
 // ctas > 0: with the smallest shared-memory carve-out that holds so many CTAs
 // (and the 1 KB that each takes on top); the rest of the SM's 256 KB is L1.
+// cluster > 1: clusters of so many CTAs along x (ctas is then 0).
 constexpr size_t kSmSmem = 228 * 1024;
 template <class A>
 inline cudaError_t launch_early(void (*fn)(A), const A& args, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                                int ctas = 0)
+                                int ctas = 0, int cluster = 1)
 {
-    cudaLaunchAttribute at[2] = {};
+    cudaLaunchAttribute at[3] = {};
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
     const size_t percent = ((smem + 1024) * ctas * 100 + kSmSmem - 1) / kSmSmem;  // rounded up
     at[1].val.sharedMemCarveout = (unsigned)(percent < 100 ? percent : 100);
+    int n_at = 1;
+    if (ctas > 0) ++n_at;
+    if (cluster > 1) {
+        at[n_at].id = cudaLaunchAttributeClusterDimension;
+        at[n_at].val.clusterDim.x = (unsigned)cluster;
+        at[n_at].val.clusterDim.y = at[n_at].val.clusterDim.z = 1;
+        ++n_at;
+    }
     cudaLaunchConfig_t c{};
     c.gridDim = grid;
     c.blockDim = dim3(threads);
     c.dynamicSmemBytes = smem;
     c.stream = st;
     c.attrs = at;
-    c.numAttrs = ctas > 0 ? 2 : 1;
+    c.numAttrs = n_at;
     return cudaLaunchKernelEx(&c, fn, args);
 }
 
@@ -232,6 +241,7 @@ struct GatherTiledArgs {
     int zs;                // z segment per CTA (divides nz, multiple of 4, <= 128)
     int rows_cap;          // largest footprint, rows
     int stages;            // footprint buffers (angles in flight + 1)
+    bool pair;             // two CTAs (a cluster) per tile and segment share the angles
     float* out;            // [batch][n][n][nz]
     int accumulate;
     UpdateSpec upd;        // as GatherArgs
@@ -287,6 +297,8 @@ cudaError_t launch_gather_tiled_tables(const float4* cs, int n, int nz, int n_an
                                        int* rows_max, int* err, cudaStream_t st);
 cudaError_t launch_gather_tiled(const GatherTiledArgs& a, cudaStream_t st);
 size_t gather_tiled_smem(int rows_cap, int zs, int T, int stages, int n_sel);  // n_sel: angles per launch
+// Whether the footprint buffers hold the sums that one CTA of a pair hands to the other.
+bool gather_pair_fits(int rows_cap, int zs, int stages);
 // Instantiations compiled in translation units of their own.
 template <int IPT, bool kHigh> cudaError_t forward_launch_ipt(const ForwardArgs& a, cudaStream_t st);
 template <int IPT, bool kHigh> int forward_occupancy_ipt(int threads, size_t smem);

@@ -459,6 +459,15 @@ int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_
                 gt.zs = p->gt_zs;
                 gt.rows_cap = p->gt_rows;
                 gt.stages = p->gt_stages;
+                // Fewer tiles than SMs: pairs of CTAs that share the angles.  96^3 x
+                // 12 angles, one subset in an OSEM run, us: 34.1 -> 27.4 with the
+                // events around it; a subset's sensitivity 28.4 -> 22.4; back of 96
+                // angles 479 -> 407.  With as many tiles as SMs or more it costs
+                // a second wave: 112^3 36.6 -> 48.6, 128^3 43.6 -> 57.7.  Blind to
+                // the batch, so that a volume is summed in the same order alone and
+                // in a batch (two volumes at 96^3 739 -> 785, three 1078 -> 1073).
+                gt.pair = ng >= 4 && p->gt_tiles * (p->nz / p->gt_zs) <= p->num_sms &&
+                          gather_pair_fits(p->gt_rows, p->gt_zs, p->gt_stages);
                 gt.out = out_b;
                 gt.accumulate = g0 > 0 || accumulate;
                 if (fused) gt.upd = *upd;
