@@ -748,11 +748,16 @@ __global__ void __launch_bounds__(kPetThreads) pet_z_kernel(LmArgs a)
 // x <- x * out / (sens / M) where sens / M > 0 (x unchanged elsewhere).
 // Blocks of 32 x 8 outputs (z, y) of one x, so that no index is divided (with
 // 64-bit divisions and one output a thread the three passes took 152 us at 204
-// x 204 x 154; without the divisions 112; with runs along x and y 92).
+// x 204 x 154; without the divisions 112; with runs along x and y 92).  Radii up
+// to kRrUnrolled have passes of their own (kR, else -1) whose taps are constants
+// of the instructions: the loop over them had cost more than its loads (with
+// the events around them 92 -> 48 us, with the update 108 -> 70).
 constexpr int kRrZ = 32, kRrY = 8;
 constexpr int kRrRun = 8;  // x and y passes: outputs of a thread along the axis, which share their inputs
 
-template <int AX>
+constexpr int kRrUnrolled = 8;
+
+template <int AX, int kR>
 __global__ void __launch_bounds__(kRrZ * kRrY) pet_rr_kernel(const float* __restrict__ in, float* __restrict__ out,
                                                              RrTaps taps, int nx, int ny, int nz,
                                                              const float* __restrict__ sens, float inv_m)
@@ -771,15 +776,28 @@ __global__ void __launch_bounds__(kRrZ * kRrY) pet_rr_kernel(const float* __rest
     for (int q = 0; q < run; ++q) acc[q] = 0.f;
     // inputs pos + m from the highest down, so that every output's sum runs
     // over its taps in rising order
-    const int hi = min(run - 1 + r, n_ax - 1 - pos), lo = max(-r, -pos);
-    const float* p = in + i + hi * st;
-#pragma unroll 4
-    for (int m = hi; m >= lo; --m, p -= st) {
-        const float v = __ldg(p);
+    if (kR >= 0) {
+        const float* p = in + i;
 #pragma unroll
-        for (int q = 0; q < run; ++q) {
-            const int t = q - m + r;
-            if (t >= 0 && t <= 2 * r) acc[q] = fmaf(taps.w[t], v, acc[q]);
+        for (int m = run - 1 + kR; m >= -kR; --m) {
+            const float v = (unsigned)(pos + m) < (unsigned)n_ax ? __ldg(p + m * st) : 0.f;
+#pragma unroll
+            for (int q = 0; q < run; ++q) {
+                const int t = q - m + kR;
+                if (t >= 0 && t <= 2 * kR) acc[q] = fmaf(taps.w[t], v, acc[q]);
+            }
+        }
+    } else {
+        const int hi = min(run - 1 + r, n_ax - 1 - pos), lo = max(-r, -pos);
+        const float* p = in + i + hi * st;
+#pragma unroll 4
+        for (int m = hi; m >= lo; --m, p -= st) {
+            const float v = __ldg(p);
+#pragma unroll
+            for (int q = 0; q < run; ++q) {
+                const int t = q - m + r;
+                if (t >= 0 && t <= 2 * r) acc[q] = fmaf(taps.w[t], v, acc[q]);
+            }
         }
     }
 #pragma unroll
@@ -936,6 +954,20 @@ int launch(pet_plan* p, const char* name, cudaStream_t st, int kernels, F&& fn)
     return SPECT_OK;
 }
 
+template <int AX>
+void launch_rr(dim3 grid, dim3 block, cudaStream_t st, const float* in, float* out, const RrTaps& taps, int nx, int ny,
+               int nz, const float* sens, float inv_m)
+{
+    switch (taps.r) {
+#define PET_RR_CASE(R) \
+    case R: pet_rr_kernel<AX, R><<<grid, block, 0, st>>>(in, out, taps, nx, ny, nz, sens, inv_m); return;
+        PET_RR_CASE(1) PET_RR_CASE(2) PET_RR_CASE(3) PET_RR_CASE(4)
+        PET_RR_CASE(5) PET_RR_CASE(6) PET_RR_CASE(7) PET_RR_CASE(kRrUnrolled)
+#undef PET_RR_CASE
+        default: pet_rr_kernel<AX, -1><<<grid, block, 0, st>>>(in, out, taps, nx, ny, nz, sens, inv_m);
+    }
+}
+
 // out = T_rr in (three passes through t1, t2), or the update of x (sens set).
 int rr_apply(pet_plan* p, const float* in, float* out, const float* sens, cudaStream_t st)
 {
@@ -945,9 +977,9 @@ int rr_apply(pet_plan* p, const float* in, float* out, const float* sens, cudaSt
     const dim3 grid0(bz, by, (nx + kRrRun - 1) / kRrRun), grid1(bz, bx, (ny + kRrRun - 1) / kRrRun), grid2(bz, by, nx);
     const float inv_m = 1.f / (float)p->geom.n_subsets;
     return launch(p, sens ? "rr_update" : "rr_blur", st, 3, [&] {
-        pet_rr_kernel<0><<<grid0, block, 0, st>>>(in, p->t1, p->taps[0], nx, ny, nz, nullptr, 0.f);
-        pet_rr_kernel<1><<<grid1, block, 0, st>>>(p->t1, p->t2, p->taps[1], nx, ny, nz, nullptr, 0.f);
-        pet_rr_kernel<2><<<grid2, block, 0, st>>>(p->t2, out, p->taps[2], nx, ny, nz, sens, inv_m);
+        launch_rr<0>(grid0, block, st, in, p->t1, p->taps[0], nx, ny, nz, nullptr, 0.f);
+        launch_rr<1>(grid1, block, st, p->t1, p->t2, p->taps[1], nx, ny, nz, nullptr, 0.f);
+        launch_rr<2>(grid2, block, st, p->t2, out, p->taps[2], nx, ny, nz, sens, inv_m);
     });
 }
 

@@ -97,3 +97,28 @@ def test_quads_em_equals_its_parts(spect_lib, cuda, shape, tof):
     assert torch.all((out - ref).abs() <= 2e-4 * ref + 1e-30)
     assert float(ref.max()) > 0.0
     plan.close()
+
+
+@pytest.mark.parametrize("radius", [1, 4, 8, 9, 14])
+@pytest.mark.parametrize("shape", [(13, 17, 35), (8, 9, 32), (3, 2, 5)])
+def test_blur_radii(spect_lib, cuda, shape, radius):
+    """T_rr on both sides of the largest unrolled radius, wider and narrower than the axes: the back projection with
+    it is the plain one blurred in float64 (2e-4: the two back projections' 1e-4, and 3 x 30 roundings)."""
+    from paper_2309_01977_gb300 import pet
+    rng = np.random.Generator(np.random.PCG64(sum(shape) + radius))
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(cuda)
+    lors = t(_lines(shape, 700, rng))
+    q = t(rng.uniform(0.1, 1.0, size=700).astype(np.float32))
+    sigma = radius / 3.0 - 0.05  # ceil(3 sigma) = radius
+    plain = pet.PetPlan(pet.PetGeometry(shape, (1.0, 1.0, 1.0)))
+    blurred = pet.PetPlan(pet.PetGeometry(shape, (1.0, 1.0, 1.0), rr_sigma_mm=sigma))
+    ref = plain.back(q, lors).cpu().numpy().astype(np.float64)
+    u = np.arange(-radius, radius + 1)
+    w = np.exp(-u ** 2 / (2.0 * float(np.float32(sigma)) ** 2))
+    w /= w.sum()
+    for ax in range(3):
+        ref = np.apply_along_axis(lambda v: np.convolve(v, w, mode="full")[radius:radius + len(v)], ax, ref)
+    got = blurred.back(q, lors).cpu().numpy()
+    assert np.all(np.abs(got - ref) <= 2e-4 * ref + 1e-30)
+    plain.close()
+    blurred.close()
