@@ -573,9 +573,8 @@ def run_pet_leg(torch, dev, timed, max_over_ranks, world, k, cpu_seconds: float,
     if os.path.exists(l2):
         with open(l2) as fh:
             prof_l2 = json.load(fh).get(em_name)
-        # the walk gathers from and scatters into an image held in L2: its
-        # bound is L2 throughput, measured by ncu as a fraction of L2 peak
-        # (with time of flight the erf weights also keep the issue slots busy)
+        # the walk gathers from and scatters into quads of the image through
+        # L2: its throughput as a fraction of L2 peak, measured by ncu
         if prof_l2:
             leg["roofline"] = {"bound": "l2", "kernel": em_name, "frac": prof_l2["lts_throughput_frac"],
                                "issue_active_frac": prof_l2["issue_active_frac"], "measured_in_run": False,

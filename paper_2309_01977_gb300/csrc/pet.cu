@@ -378,12 +378,15 @@ __global__ void __launch_bounds__(kPetThreads) pet_lm_kernel(LmArgs a)
 // per voxel afterwards.  The lines of one axis go together (x, then y), so
 // that one axis's quads are in use at a time; lines along z, which a
 // cylindrical scanner hardly has, walk the image.
-// Bound by L1's rate of one line a cycle.  With a line of response to a lane
-// and cells in plane order, a warp's 32 lanes touched 32 lines a sample each
-// way (1.7 cycles a sample for the gather, 2.0 for the scatter).  Four lanes
+// With a line of response to a lane and cells in plane order the walk was bound
+// by L1's rate of one line a cycle: a warp's 32 lanes touched 32 lines a sample
+// each way (1.7 cycles a sample for the gather, 2.0 for the scatter).  Four lanes
 // now walk a line together, on consecutive planes, and the cells lie in
 // 128-byte bricks of 4 planes x 2 u x 1 w, so that the four share about two
-// lines (along the axis a line moves by half a cell in u and less in w).
+// lines (along the axis a line moves by half a cell in u and less in w).  What
+// bounds it now is the latency of misses past L2: at 204 x 204 x 154 the two sets
+// of quads are 104 MB each, 43 % of the sectors hit, and HBM moves 3.8 TB/s; L1
+// and the issue slots are half busy.
 // Measured, image walk -> quads in plane order -> bricks: an iteration of 3 M
 // events in 3 subsets at 204 x 204 x 154 with time of flight 9.7 -> 6.95 ->
 // 5.58 ms; 128 x 128 x 90, 1 M lines without, forward and back 2.60 -> 1.46 ->
