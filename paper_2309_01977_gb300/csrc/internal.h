@@ -98,7 +98,9 @@ inline cudaError_t launch_early(void (*fn)(A), const A& args, dim3 grid, int thr
     c.stream = st;
     c.attrs = at;
     c.numAttrs = n_at;
-    return cudaLaunchKernelEx(&c, fn, args);
+    const cudaError_t e = cudaLaunchKernelEx(&c, fn, args);
+    if (e != cudaSuccess) cudaGetLastError();  // do not leave the failure to a later launch check
+    return e;
 }
 
 // threads % width and threads / width of a grid of items, `width` to a row.

@@ -1006,11 +1006,11 @@ int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream,
     // of footprint rows is one contiguous copy), longer ones in equal segments
     // of 80 to 128 where there are such, and two footprint buffers (one angle
     // in flight; a third buffer measured slower on GB300).  Else the
-    // per-column gather.  Tiled against per column, one subset, us: 64^3 x 8
-    // angles 19.6 / 12.3, 77 x 77 x 100 x 15 33.6 / 33.1, 96^3 x 12 26.7 /
-    // 32.9, 96^3 x 16 x 2 volumes 40.7 / 89.3, 112^3 x 12 31 / 49, 160^3 x 8
-    // (two segments of 80) 89 / 121, 192^3 x 16 (two of 96) 222 / 313, in
-    // three of 64 318.
+    // per-column gather.  Tiled against per column, one subset with the events
+    // around it, us: 64^3 x 8 angles 21.6 / 12.2, 80 x 80 x 64 x 8 22.5 / 22.5
+    // (a whole iteration 487 / 466), 96^3 x 12 27.4 (pairs) / 39.4, 112 x 112 x
+    // 96 x 12 36.6 / 58.2; launches alone: 160^3 x 8 (two segments of 80) 89 /
+    // 121, 192^3 x 16 (two of 96) 222 / 313, in three of 64 318.
     int zs = p->nz <= 128 ? p->nz : 0;
     for (int d = 2; zs == 0 && p->nz / d >= 80; ++d)
         if (p->nz % (4 * d) == 0 && p->nz / d <= 128) zs = p->nz / d;
