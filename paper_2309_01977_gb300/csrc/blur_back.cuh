@@ -249,7 +249,7 @@ cudaError_t launch_sq(const BlurBackArgs& a, cudaStream_t st)
     cudaError_t e = allow_big_smem(blur_back_kernel<kSq, kSmemA, kHigh>, g_blur_back_smem_mask<kSq, kSmemA, kHigh>);
     if (e != cudaSuccess) return e;
     const dim3 grid(a.chunks * a.t.ntiles, a.n_sel, a.batch);
-    return launch_early(blur_back_kernel<kSq, kSmemA, kHigh>, a, grid, a.t.threads, a.t.smem, st);
+    return launch_early(blur_back_kernel<kSq, kSmemA, kHigh>, a, grid, a.t.threads, a.t.smem, st, 0, 1, a.early);
 }
 
 template <int kSq, bool kSmemA, bool kHigh>

@@ -64,27 +64,36 @@ constexpr int kBackStrides[] = {9, 17, 33, 49, 65};  // strides of Q: half a til
 // kernels of the stream write or read: its CTAs may take their SMs while the
 // last CTAs of the kernel before it still run, so that the launch and the part
 // of the kernel that needs only plan data (tables, barriers, shared-memory
-// zeros, the first attenuation plane) overlap that kernel's tail.  After any
-// other kernel or copy it starts as an ordinary launch does.  Measured, OSEM
+// zeros, the first attenuation plane) overlap that kernel's tail.  After a
+// kernel without launch_dependents() its CTAs may start once that kernel's
+// blocks have ended, and what those wrote is visible past
+// wait_prerequisites() only: a launch that reads plan data ahead of the wait
+// has early false where the kernel before it wrote that data.  Measured, OSEM
 // with ordinary and with early launches: 64^3, 16 subiterations of 8 angles
 // 741 -> 654 us (BF16, 8 subiterations 467 -> 390); 96^3 x 12 x 8 968 -> 907;
 // 128^3 x 15 x 8 1766 -> 1717 (BF16 1430 -> 1400).
 // ctas > 0: with the smallest shared-memory carve-out that holds so many CTAs
 // (and the 1 KB that each takes on top); the rest of the SM's 256 KB is L1.
 // cluster > 1: clusters of so many CTAs along x (ctas is then 0).
+// early false: an ordinary launch, after all that came before it in the stream.
 constexpr size_t kSmSmem = 228 * 1024;
 template <class A>
 inline cudaError_t launch_early(void (*fn)(A), const A& args, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                                int ctas = 0, int cluster = 1)
+                                int ctas = 0, int cluster = 1, bool early = true)
 {
     cudaLaunchAttribute at[3] = {};
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    const size_t percent = ((smem + 1024) * ctas * 100 + kSmSmem - 1) / kSmSmem;  // rounded up
-    at[1].val.sharedMemCarveout = (unsigned)(percent < 100 ? percent : 100);
-    int n_at = 1;
-    if (ctas > 0) ++n_at;
+    int n_at = 0;
+    if (early) {
+        at[n_at].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n_at].val.programmaticStreamSerializationAllowed = 1;
+        ++n_at;
+    }
+    if (ctas > 0) {
+        const size_t percent = ((smem + 1024) * ctas * 100 + kSmSmem - 1) / kSmSmem;  // rounded up
+        at[n_at].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[n_at].val.sharedMemCarveout = (unsigned)(percent < 100 ? percent : 100);
+        ++n_at;
+    }
     if (cluster > 1) {
         at[n_at].id = cudaLaunchAttributeClusterDimension;
         at[n_at].val.clusterDim.x = (unsigned)cluster;
@@ -173,6 +182,7 @@ struct BlurBackArgs {
     int n, nz, n_sel, batch;
     int chunks;            // depth chunks: contiguous plane ranges of equal work
     BackTiling t;
+    bool early;            // launch_early; false where the kernel before has written atten
     float* bvol;           // [batch][n_sel][n][n][nz] rotated-frame volumes A . (K_i r)
     int* err;              // SPECT_ETIMEDOUT when a bounded wait runs out
 };

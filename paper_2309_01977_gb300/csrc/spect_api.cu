@@ -369,8 +369,9 @@ int run_forward(spect_plan* p, spect_plan_scratch& sc, const float* x, float* ou
 
 // x_out (per batch entry) = sum over sel of H_a^T proj_a, optionally fused with
 // the OSEM update x_out <- x_out * bp / sens (then batch must be 1).
+// atten_new: the last kernel queued on st is the one that writes A_a.
 int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_out, const int* sel_dev, int n_sel,
-             int batch, const UpdateSpec* upd, cudaStream_t st, bool accumulate = false)
+             int batch, const UpdateSpec* upd, cudaStream_t st, bool accumulate = false, bool atten_new = false)
 {
     const size_t vol = vol_elems(p), plane = plane_elems(p);
     const int gmax = (int)std::min<size_t>(kGatherMaxAngles, p->bvol_cap);
@@ -439,6 +440,9 @@ int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_
                 bb.batch = nb;
                 bb.t = p->back;
                 bb.chunks = chunk_target(p, (long)nb * ng * p->back.ntiles, p->back_occ);
+                // its first plane of A is copied ahead of the wait; the later
+                // launches of this call come after one that has waited
+                bb.early = !(atten_new && b0 == 0 && g0 == 0);
                 bb.bvol = sc.bvol;
                 bb.err = p->d_err;
                 e = timed(p, "blur_back", st, 1, [&] { return launch_blur_back(bb, st); });
@@ -761,7 +765,7 @@ int refresh_mu(spect_plan* p, spect_plan_scratch& sc, const float* mu_dev, cudaS
     }
     for (int m = 0; m < p->M; ++m) {
         const int rc = run_back(p, sc, nullptr, p->d_sens + (size_t)m * vol, p->d_sel[m], (int)p->subsets[m].size(),
-                                1, nullptr, st);
+                                1, nullptr, st, false, m == 0);
         if (rc) return rc;
     }
     return SPECT_OK;
