@@ -11,14 +11,14 @@ namespace {
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-// Forward z tile of ktile columns; smem 0 where its strips do not fit.
-PlaneTiling make_tiling(int n, int nz, int rmax, int ktile, size_t cap, size_t limit)
+// Forward z tile of ktile columns, its halo a multiple of `halo`; smem 0 where
+// its strips do not fit.
+PlaneTiling make_tiling(int n, int nz, int rmax, int ktile, int halo, size_t cap, size_t limit)
 {
     PlaneTiling t{};
     t.ktile = ktile;
     t.ntiles = (nz + ktile - 1) / ktile;
-    // even; a multiple of 4 keeps the staged window of a tile 16-byte aligned
-    t.rh = round_up(rmax, t.ntiles > 1 ? 4 : 2);
+    t.rh = round_up(rmax, t.ntiles > 1 ? halo : 2);
     t.ktpad = round_up(ktile, kStrip);
     t.npad = round_up(n, kStrip);
     t.sp = ((t.ktpad + 2 * t.rh) / 2) | 1;
@@ -75,21 +75,25 @@ long staged_columns(const PlaneTiling& t, int nz)
 // 96-column tiles with two strips per thread: 1.25 vs 1.51 ms (384 threads)
 // and 1.77 ms (288) per launch of 16 angles and two volumes; at 160^3 two
 // 80-column tiles beat three of 64, 172 vs 233 us for 8 angles.
+// The halo of tiles is a multiple of 4, which keeps a staged window 16-byte
+// aligned, or even where no tile fits with that (planes of n = 689 to 720 with
+// radius 17 or 18).
 PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit)
 {
     PlaneTiling best{};
     double best_cost = 0;
-    for (int nt = 1; nt <= (nz + kStrip - 1) / kStrip; ++nt) {
-        const int kt = nt == 1 ? nz : round_up((nz + nt - 1) / nt, kStrip);
-        if (nt > 1 && (nt - 1) * kt >= nz) continue;  // same as a smaller count
-        const PlaneTiling t = make_tiling(n, nz, rmax, kt, cap, limit);
-        if (t.smem == 0) continue;
-        const double cost = (double)staged_columns(t, nz) * (t.ipt > 1 ? 1.5 : 1.0);
-        if (best.smem == 0 || cost < best_cost) {
-            best = t;
-            best_cost = cost;
+    for (int halo = 4; halo >= 2 && best.smem == 0; halo -= 2)
+        for (int nt = 1; nt <= (nz + kStrip - 1) / kStrip; ++nt) {
+            const int kt = nt == 1 ? nz : round_up((nz + nt - 1) / nt, kStrip);
+            if (nt > 1 && (nt - 1) * kt >= nz) continue;  // same as a smaller count
+            const PlaneTiling t = make_tiling(n, nz, rmax, kt, halo, cap, limit);
+            if (t.smem == 0) continue;
+            const double cost = (double)staged_columns(t, nz) * (t.ipt > 1 ? 1.5 : 1.0);
+            if (best.smem == 0 || cost < best_cost) {
+                best = t;
+                best_cost = cost;
+            }
         }
-    }
     return best;  // smem == 0: does not fit
 }
 
