@@ -97,26 +97,32 @@ PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit)
     return best;  // smem == 0: does not fit
 }
 
-// Back blur.  Among the tile widths that fit: the fewest rounds of strips per
-// plane, a CTA of 256 threads (two to an SM) counted half; then the widest
-// tile.  The CTA has 256 threads where a pass over a plane has that many
-// strips or fewer, else 512, and the attenuation comes through shared memory
-// where a tile is the whole plane and the buffer fits.  Measured (one subset,
-// us): 64^3 x 8 angles 256 threads 14.6, two 32-column tiles of 256 16.1;
-// 96^3 x 12 one tile of 512 threads 36.8, two of 256 43.6; 128^3 x 15 one
-// tile of 512 87, two of 256 86; 132 x 44 x 16 256 threads 47.5 (A from global
-// memory 51.3); 160^3 x 8 two tiles of 96 columns 116, five of 32 126; 192^3
-// x 16 x 2 volumes three tiles of 64 columns 332, two of 96 402, six of 32
-// 351; 77 x 77 x 100 x 15 A through shared memory 33.5, from global 65.
+// Back blur.  Among the tile widths that fit, each with the narrowest stride of
+// kBackStrides that holds it: the fewest rounds of strips per plane, a round of
+// 256 threads counted half; then the widest tile.  The CTA has 256 threads
+// where a pass over a plane has that many strips or fewer and two such CTAs fit
+// an SM, else 512, and the attenuation comes through shared memory where a tile
+// is the whole plane and the buffer fits.  Measured (one subset, us): 64^3 x 8
+// angles 256 threads 14.3, two 32-column tiles of 256 16.3; 96^3 x 12 one tile
+// of 512 threads 39.8, two of 256 47.2; 128^3 x 15 one tile of 512 87, two of
+// 256 85; 160^3 x 8 two tiles of 96 columns 117, three of 64 131; 192^3 x 16 x
+// 2 volumes three tiles of 64 columns 338, two of 96 406.  A wider stride than
+// the tile needs takes the second CTA or the attenuation buffer: 132 x 44 x 15
+// stride 33 two CTAs 47.4, 65 one of 256 threads 54.5, one of 512 51.8; 80 x 96
+// x 12 stride 49 two CTAs 24.9, 65 one of 256 28.6, one of 512 26.7; 190 x 56 x
+// 12 stride 33 with the buffer 103, 65 without 173.
 BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit)
 {
     BackTiling best{};
     double best_cost = 0.0;
+    int last_width = 0;
     const int npad = round_up(n, kStrip), rp = npad / 2, rh = rmax + (rmax & 1);
     for (int sq : kBackStrides) {
         BackTiling t{};
         t.sq = sq;
         t.ktpad = std::min(2 * (sq - 1), round_up(nz, kStrip));
+        if (t.ktpad == last_width) break;  // this stride and the wider ones add padding only
+        last_width = t.ktpad;
         t.ktile = std::min(t.ktpad, nz);
         t.ntiles = (nz + t.ktile - 1) / t.ktile;
         t.rh = rh;
@@ -137,7 +143,8 @@ BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit)
         t.smem_a = atten && t.ntiles == 1 && with_a <= limit;  // a tile's rows would be copied one by one
         t.smem = t.smem_a ? with_a : bare;
         if (t.smem > limit) continue;
-        const int thr = std::max(zitems, jitems) <= kPlaneThreads / 2 ? kPlaneThreads / 2 : kPlaneThreads;
+        const bool two = 2 * (t.smem + 1024) <= kSmSmem;
+        const int thr = two && std::max(zitems, jitems) <= kPlaneThreads / 2 ? kPlaneThreads / 2 : kPlaneThreads;
         t.threads = thr;
         t.zstep = {thr % rp, thr / rp};
         t.jstep = {thr % (t.ktpad / 2), thr / (t.ktpad / 2)};

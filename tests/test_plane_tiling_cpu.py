@@ -73,3 +73,26 @@ def test_planes_that_fit_are_accepted(tilings):
             assert 0 < t["smem"] <= LIMIT and t["f_smem"] <= LIMIT, (n, nz, r)
         took, refused = took + fits, refused + (not fits)
     assert took > 100 and refused > 100
+
+
+def test_back_tilings_carry_no_padding(tilings):
+    """The back blur's stride is the narrowest that holds its tile, a CTA of 256
+    threads is one of two that fit an SM, and a whole plane's attenuation is
+    staged where the buffer fits."""
+    strides = (9, 17, 33, 49, 65)  # kBackStrides
+    shapes = [(n, nz, r, 1) for n in range(32, 193, 3) for nz in range(24, 193, 4) for r in (3, 9, 15, 19)]
+    halved = staged = 0
+    for (n, nz, r, _), t in zip(shapes, tilings(shapes)):
+        assert t["smem"] > 0, (n, nz, r)
+        width = min(s for s in strides if min(2 * (s - 1), _up(nz, 16)) == t["ktpad"])
+        assert t["sq"] == width, (n, nz, r, t)
+        assert t["threads"] in (256, 512)
+        if t["threads"] == 256:
+            assert 2 * (t["smem"] + 1024) <= 228 * 1024, (n, nz, r, t)
+            halved += 1
+        rp, rh = _up(n, 16) // 2, _up(r, 2)
+        bare = 16 * (rp * ((t["ktpad"] + 2 * rh) // 2 | 1) + (rp + 2 * ((r + 1) // 2)) * t["sq"]) + 2 * 21 * 4
+        fits = t["ntiles"] == 1 and _up(bare, 16) + 4 * n * nz + 8 <= LIMIT
+        assert t["smem_a"] == fits, (n, nz, r, t)
+        staged += fits
+    assert halved > 100 and staged > 100
