@@ -107,44 +107,95 @@ cudaError_t launch_attenuation(const float* mu, const float4* cs, int n, int nz,
     return cudaGetLastError();
 }
 
-// Rotated-frame volumes of all-ones projections (the sensitivities H_m^T 1):
-// the blur of a constant is the outer product of the taps' partial sums at
-// the plane's edges, so B_a[i][j][k] = A_a[i][j][k] v_i(j) w_i(k) with
-// v_i(j) = sum of w_i(t) over 0 <= j - t < n, and w_i(k) alike over nz.  One
-// block per (plane, angle); bound by the HBM traffic of A and B where the
-// blur of every plane was bound by its FMAs (96^3 x 12 angles: see launch).
+// Rotated-frame volumes of all-ones projections (the sensitivities H_m^T 1).
+// The blur of a constant depends only on how far a bin lies from the plane's
+// edges, so min(n, 2R + 1) x min(nz, 2R + 1) sums a plane hold every value of
+// it; they run over the taps as the strips of blur_back.cuh do, in the same
+// order with the same roundings, so that B has the bits of the blur kernel and
+// an update's ratio cancels the rounding that both of its back projections
+// share.  One block per (plane, angle); bound by the HBM traffic of A and B where
+// the blur of every plane was bound by its FMAs.
+// Closed form v_i(j) w_i(k) of the same sums in its place: no faster, and images
+// further from 64 bits (64^3 x 64 angles, 2 x 8 subsets: 8.1e-7, with the blur's
+// bits 7.9e-7).
+__device__ __forceinline__ int edge_class(int pos, int m, int R) { return max(min(pos, R), pos - max(m - 1 - 2 * R, 0)); }
+
+// A position of class c among m.
+__device__ __forceinline__ int class_pos(int c, int m, int R) { return c <= R ? c : c + max(m - 1 - 2 * R, 0); }
+
+constexpr int kOnesTaps = (kTapW + 3) / 4 * 4;
+
 __global__ void __launch_bounds__(256) ones_back_kernel(BlurBackOnesArgs a)
 {
-    extern __shared__ float edge[];  // v_i [n], w_i [nz]
+    extern __shared__ __align__(16) int at[];  // class of every column [nz], first sum of every row's class [n]
+    // the plane's taps, zero past them (a product with 0 adds nothing), so that
+    // the sums run over whole float4
+    __shared__ float4 w4[kOnesTaps / 4];
+    __shared__ float zsum[kTapW], val[kTapW * kTapW];
     const int i = blockIdx.x, sidx = blockIdx.y, n = a.n, nz = a.nz;
     const int angle = a.sel[sidx];
     const float* taps = a.taps + (size_t)angle * a.taps_stride + (size_t)i * kTapW + kMaxR;
     const int R = a.rad[(size_t)angle * a.rad_stride + i];
-    for (int e = threadIdx.x; e < n + nz; e += blockDim.x) {
-        const int m = e < n ? n : nz, pos = e < n ? e : e - n;
+    const int cn = min(n, 2 * R + 1), cz = min(nz, 2 * R + 1), groups = (2 * R + 4) / 4;
+    if (threadIdx.x < kOnesTaps)
+        reinterpret_cast<float*>(w4)[threadIdx.x] = threadIdx.x <= 2 * R ? __ldg(taps + ((int)threadIdx.x - R)) : 0.f;
+    for (int e = threadIdx.x; e < nz + n; e += blockDim.x)
+        at[e] = e < nz ? edge_class(e, nz, R) : edge_class(e - nz, n, R) * cz;
+    __syncthreads();
+    if (threadIdx.x < cz) {
+        // tap u reaches column k - R + u
+        const int k = class_pos(threadIdx.x, nz, R), lo = R - k, hi = R + nz - 1 - k;
         float s = 0.f;
-        for (int t = max(-R, pos - (m - 1)); t <= min(R, pos); ++t) s += __ldg(taps + t);
-        edge[e] = s;
+#pragma unroll 4
+        for (int g = 0; g < groups; ++g) {
+            const float4 w = w4[g];
+            const int u = 4 * g;
+            s = __fadd_rn(s, u >= lo && u <= hi ? w.x : 0.f);
+            s = __fadd_rn(s, u + 1 >= lo && u + 1 <= hi ? w.y : 0.f);
+            s = __fadd_rn(s, u + 2 >= lo && u + 2 <= hi ? w.z : 0.f);
+            s = __fadd_rn(s, u + 3 >= lo && u + 3 <= hi ? w.w : 0.f);
+        }
+        zsum[threadIdx.x] = s;
     }
     __syncthreads();
-    const int zq = nz >> 2;
+    for (int e = threadIdx.x; e < cn * cz; e += blockDim.x) {
+        const int c = e / cz, j = class_pos(c, n, R), lo = R - j, hi = R + n - 1 - j;
+        const float z = zsum[e - c * cz];
+        float s = 0.f;
+#pragma unroll 4
+        for (int g = 0; g < groups; ++g) {
+            const float4 w = w4[g];
+            const int u = 4 * g;
+            s = __fmaf_rn(w.x, u >= lo && u <= hi ? z : 0.f, s);
+            s = __fmaf_rn(w.y, u + 1 >= lo && u + 1 <= hi ? z : 0.f, s);
+            s = __fmaf_rn(w.z, u + 2 >= lo && u + 2 <= hi ? z : 0.f, s);
+            s = __fmaf_rn(w.w, u + 3 >= lo && u + 3 <= hi ? z : 0.f, s);
+        }
+        val[e] = s;
+    }
+    __syncthreads();
+    const int zq = nz >> 2, dj = blockDim.x / zq, dk = blockDim.x - dj * zq;
     const float4* A = a.atten ? reinterpret_cast<const float4*>(a.atten + ((size_t)angle * n + i) * n * nz) : nullptr;
     float4* B = reinterpret_cast<float4*>(a.bvol + ((size_t)sidx * n + i) * n * nz);
+    int j = threadIdx.x / zq, k = threadIdx.x - j * zq;
+#pragma unroll 4
     for (int e = threadIdx.x; e < n * zq; e += blockDim.x) {
-        const int j = e / zq, k = 4 * (e - j * zq);
-        const float v = edge[j];
-        float4 b = make_float4(v * edge[n + k], v * edge[n + k + 1], v * edge[n + k + 2], v * edge[n + k + 3]);
-        if (A) {
-            const float4 q = __ldg(A + e);
-            b = make_float4(b.x * q.x, b.y * q.y, b.z * q.z, b.w * q.w);
+        const int4 c = reinterpret_cast<const int4*>(at)[k];
+        const float* v = val + at[nz + j];
+        const float4 q = A ? __ldg(A + e) : make_float4(1.f, 1.f, 1.f, 1.f);
+        B[e] = make_float4(v[c.x] * q.x, v[c.y] * q.y, v[c.z] * q.z, v[c.w] * q.w);
+        j += dj;
+        k += dk;
+        if (k >= zq) {
+            k -= zq;
+            ++j;
         }
-        B[e] = b;
     }
 }
 
 cudaError_t launch_blur_back_ones(const BlurBackOnesArgs& a, cudaStream_t st)
 {
-    ones_back_kernel<<<dim3(a.n, a.n_sel), 256, (size_t)(a.n + a.nz) * sizeof(float), st>>>(a);
+    ones_back_kernel<<<dim3(a.n, a.n_sel), 256, (size_t)(a.n + a.nz) * sizeof(int), st>>>(a);
     return cudaGetLastError();
 }
 
