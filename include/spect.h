@@ -218,7 +218,8 @@ int spect_osem_run_dev(spect_plan* plan, const float* y, const float* s_dev, flo
  *   SPECT_PRIOR_QUADRATIC  phi = ((a - b) / delta)^2 / 4
  *   SPECT_PRIOR_RDP        phi = (a - b)^2 / (a + b + gamma |a - b|)
  *                          (relative difference prior; a pair whose
- *                          denominator is 0 contributes 0). */
+ *                          denominator is 0, or no normal float, contributes
+ *                          0). */
 #define SPECT_PRIOR_NONE 0
 #define SPECT_PRIOR_QUADRATIC 1
 #define SPECT_PRIOR_RDP 2

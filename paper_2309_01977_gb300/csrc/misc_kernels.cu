@@ -1,6 +1,8 @@
 // Attenuation cache, FP64 count reductions and the Poisson likelihood.
 #include <cuda_runtime.h>
 
+#include <cfloat>
+
 #include "async_copy.cuh"
 #include "geometry.cuh"
 #include "internal.h"
@@ -439,6 +441,8 @@ cudaError_t launch_wsum(float* out, const float* const* in, const float* w, int 
 //   RDP  phi = (a - b)^2 / (a + b + gamma|a - b|):
 //        dphi/da = (a - b)(a + 3b + gamma|a - b|) / (a + b + gamma|a - b|)^2,
 //   a pair whose RDP denominator is 0 contributing 0.
+// So does a pair whose S (below) is subnormal: 1 / S is past the largest float
+// there, and two equal neighbours would give 0 inf.
 // A thread walks kPriorRun voxels along i, z fastest over the lanes, with the
 // 27 values around its voxel in registers (nine loads a voxel).  Bound by the
 // RDP's arithmetic, 26 terms a voxel: with S the denominator's root, a term is
@@ -497,7 +501,7 @@ __global__ void __launch_bounds__(kPriorZ * kPriorJ) prior_grad_kernel(const flo
                 if (kRdp) {
                     const float S = fmaf(gamma, fabsf(d), a + b), q = __frcp_rn(S);
                     t = (d * q) * (fmaf(2.f, b, S) * q);
-                    ok = ok && S != 0.f;
+                    ok = ok && !(fabsf(S) < FLT_MIN);
                 }
                 g = fmaf(w, ok ? t : 0.f, g);
             }
