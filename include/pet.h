@@ -44,8 +44,15 @@
  *
  * Memory: every pointer argument is a device pointer (the caller owns it) to
  * contiguous FP32 data, LOR arrays 8-byte aligned, images 16-byte aligned;
- * diag_out is a host pointer.  The plan owns its taps, a copy of mu and its
- * scratch images.  Calls are asynchronous on `stream` (a cudaStream_t, NULL
+ * diag_out is a host pointer.  The plan owns its taps, a copy of mu, its
+ * scratch images and, from the first call with at least one line per 32
+ * voxels on, the image's quads (pet_forward, pet_lm_osem_run) and the back
+ * projection's (pet_back, pet_lm_osem_run): 16 bytes a cell of nx x ny x nz
+ * cells each (axes rounded up to the walk's bricks; 104 MB at 204 x 204 x 154).
+ * That first call allocates them, which may wait for the device, under stream
+ * capture as well, if they take half of the free memory at most; where it
+ * cannot, it projects without them and a later call tries again.  They are
+ * given back with the plan.  Calls are asynchronous on `stream` (a cudaStream_t, NULL
  * for the legacy stream) and a plan serves one stream at a time.
  * Errors: SPECT_OK (0) or a negative status of spect.h; the message is in
  * spect_last_error().  Floating-point sums that scatter (P_Sigma^T) use
@@ -77,7 +84,8 @@ typedef struct pet_geom {
 typedef struct pet_plan pet_plan;
 
 /* Plan: geometry, T_rr taps, a copy of mu (NULL: no attenuation) and the
- * scratch images (4 images of nx*ny*nz floats). */
+ * scratch images (4 images of nx*ny*nz floats; the quads of calls with many
+ * lines come later, see above). */
 int pet_plan_create(const pet_geom* geom, const float* mu_dev, void* stream, pet_plan** out);
 int pet_plan_destroy(pet_plan* plan);
 

@@ -885,8 +885,7 @@ struct pet_plan {
     float* fb = nullptr;
     float* bp = nullptr;
     float4* quads = nullptr;   // the walked image's quads of one axis, and the back projection's
-    float4* bquads = nullptr;  // (both allocated by the first call that has enough lines)
-    bool quads_failed = false; // not enough memory for them: the image is walked
+    float4* bquads = nullptr;  // (each allocated by the first call that walks it)
     double* diag = nullptr;
     int diag_cap = 0;  // subiterations the diag buffer holds
     std::vector<void*> allocations;
@@ -999,35 +998,64 @@ LmArgs base_args(const pet_plan* p, const float* lors, long long n)
     return a;
 }
 
-// Whether a call walks quads: at least one line per 32 voxels (building,
-// clearing and folding quads moves about 100 bytes a voxel and axis, some 0.1
-// ms at 204 x 204 x 154, which a line's saving of about 1 ns repays from 0.1 M
-// lines, 1 / 64 of the voxels, on), lattices that 32-bit indexes reach, and the memory for
-// them, taken once per plan (a call under stream capture takes none, and
-// where there is none the image is walked as before).
-bool use_quads(pet_plan* p, long long lines, cudaStream_t st)
+// Relaxed capture mode in this thread while it lives: a call under stream
+// capture, or next to another thread's capture, may allocate.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    bool ok;
+    RelaxedCapture() : ok(cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess)
+    {
+        if (!ok) cudaGetLastError();
+    }
+    ~RelaxedCapture()
+    {
+        if (ok) cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+};
+
+// Allocates those of the plan's quads that are wanted and missing: all of them,
+// or none where they would take more than half of the free memory (which other
+// users of the device want too) or the allocation fails.
+bool take_quads(pet_plan* p, bool image, bool back, size_t bytes)
 {
-    const long long cells = std::max(quad_cells(p->grid, 0), quad_cells(p->grid, 1));
-    if (lines < p->voxels / 32 || cells >= (1ll << 31) - (1ll << 23) || p->voxels >= (1ll << 31) || p->quads_failed) return false;
-    if (p->quads && p->bquads) return true;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    float4** want[2] = {image && !p->quads ? &p->quads : nullptr, back && !p->bquads ? &p->bquads : nullptr};
+    const size_t missing = bytes * ((want[0] ? 1 : 0) + (want[1] ? 1 : 0));
+    if (missing == 0) return true;
+    RelaxedCapture relaxed;
+    if (!relaxed.ok) return false;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    if (cap != cudaStreamCaptureStatusNone) return false;
-    for (float4** b : {&p->quads, &p->bquads}) {
-        if (*b) continue;
-        void* ptr = nullptr;
-        if (cudaMalloc(&ptr, (size_t)cells * sizeof(float4)) != cudaSuccess) {
+    if (missing > free_b / 2) return false;
+    void* got[2] = {nullptr, nullptr};
+    for (int i = 0; i < 2; ++i)
+        if (want[i] && cudaMalloc(&got[i], bytes) != cudaSuccess) {
             cudaGetLastError();
-            p->quads_failed = true;
+            cudaFree(got[0]);
             return false;
         }
-        p->allocations.push_back(ptr);
-        *b = static_cast<float4*>(ptr);
-    }
+    for (int i = 0; i < 2; ++i)
+        if (want[i]) {
+            p->allocations.push_back(got[i]);
+            *want[i] = static_cast<float4*>(got[i]);
+        }
     return true;
+}
+
+// Whether a call walks quads: at least one line per 32 voxels (building,
+// clearing and folding quads moves about 100 bytes a voxel and axis, some 0.1
+// ms at 204 x 204 x 154, which a line's saving of about 1 ns repays from 0.1 M
+// lines, 1 / 64 of the voxels, on), lattices that 32-bit indexes reach, and the
+// memory for the sets that the mode needs, kept by the plan.  Where there is
+// none the image is walked, and a later call tries again.
+template <int kMode>
+bool use_quads(pet_plan* p, long long lines)
+{
+    const long long cells = std::max(quad_cells(p->grid, 0), quad_cells(p->grid, 1));
+    if (lines < p->voxels / 32 || cells >= (1ll << 31) - (1ll << 23) || p->voxels >= (1ll << 31)) return false;
+    return take_quads(p, kMode != kModeBack, kMode != kModeFwd, (size_t)cells * sizeof(float4));
 }
 
 constexpr int kQuadBlocks = 152 * 8;  // pet_quad_kernel: every resident CTA
@@ -1052,7 +1080,7 @@ void launch_quad_axis(pet_plan* p, const LmArgs& a, cudaStream_t st)
 template <int kMode>
 int launch_walk(pet_plan* p, const char* name, LmArgs a, cudaStream_t st)
 {
-    const bool quads = use_quads(p, a.count, st);
+    const bool quads = use_quads<kMode>(p, a.count);
     const int kernels = !quads ? 1 : kMode == kModeEm ? 7 : 5;
     return launch(p, name, st, kernels, [&] {
         if (quads) {
