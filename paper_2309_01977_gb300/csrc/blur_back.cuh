@@ -270,7 +270,8 @@ int blocks_sq(const BackTiling& t)
 // instantiation per row stride of kBackStrides.
 #define SPECT_SQ_CASES(M)                                                                                     \
     case kBackStrides[0]: M(0); case kBackStrides[1]: M(1); case kBackStrides[2]: M(2);                       \
-    case kBackStrides[3]: M(3); case kBackStrides[4]: M(4)
+    case kBackStrides[3]: M(3); case kBackStrides[4]: M(4); case kBackStrides[5]: M(5);                       \
+    case kBackStrides[6]: M(6)
 
 template <bool kSmemA, bool kHigh>
 cudaError_t launch_blur_back_v(const BlurBackArgs& a, cudaStream_t st)

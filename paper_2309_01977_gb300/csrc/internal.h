@@ -44,7 +44,7 @@ struct PlaneTiling {
     int npad;     // n rounded up to kStrip
     int sp;       // P stride between row pairs, in 16-byte quads (odd): >= (ktpad + 2*rh) / 2
     int sq;       // Q stride between column pairs, in quads (odd): >= (npad + 2*rh) / 2
-    int threads;  // CTA size (multiple of 32, <= kFwdThreads)
+    int threads;  // CTA size (multiple of 32, <= kPlaneThreads)
     int ipt;      // j-blur strips per thread (1..kMaxIpt)
     int ctas;     // CTAs an SM holds (1 or 2)
     bool high;    // radii past kLowR, or several strips per thread: the kernel with every radius
@@ -56,8 +56,8 @@ struct PlaneTiling {
     size_t smem;  // dynamic shared memory: P, Q, the tap-row table, the tap buffer, the attenuation buffer
 };
 
-// Shape of one back blur launch (blur_back.cuh).
-constexpr int kBackStrides[] = {9, 17, 33, 49, 65};  // strides of Q: half a tile's columns, rounded up to odd
+// Strides of the back blur's Q: half of a tile's columns, rounded up to odd.
+constexpr int kBackStrides[] = {9, 17, 33, 49, 65, 81, 97};
 
 // Launch of a kernel that calls launch_dependents() at its start and
 // wait_prerequisites() (async_copy.cuh) before it touches what earlier
@@ -117,6 +117,7 @@ struct ItemStep {
     int dc, dr;
 };
 
+// Shape of one back blur launch (blur_back.cuh).
 struct BackTiling {
     int ktile, ntiles;  // as above
     int rh;             // halo = largest PSF radius, rounded up to even

@@ -97,34 +97,42 @@ PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit)
     return best;  // smem == 0: does not fit
 }
 
-// Back blur.  Among the tile widths that fit, each with the narrowest stride of
-// kBackStrides that holds it: the fewest rounds of strips per plane, a round of
-// 256 threads counted half; then the widest tile.  The CTA has 256 threads
-// where a pass over a plane has that many strips or fewer and two such CTAs fit
-// an SM, else 512, and the attenuation comes through shared memory where a tile
-// is the whole plane and the buffer fits.  Measured (one subset, us): 64^3 x 8
-// angles 256 threads 14.3, two 32-column tiles of 256 16.3; 96^3 x 12 one tile
-// of 512 threads 39.8, two of 256 47.2; 128^3 x 15 one tile of 512 87, two of
-// 256 85; 160^3 x 8 two tiles of 96 columns 117, three of 64 131; 192^3 x 16 x
-// 2 volumes three tiles of 64 columns 338, two of 96 406.  A wider stride than
-// the tile needs takes the second CTA or the attenuation buffer: 132 x 44 x 15
-// stride 33 two CTAs 47.4, 65 one of 256 threads 54.5, one of 512 51.8; 80 x 96
-// x 12 stride 49 two CTAs 24.9, 65 one of 256 28.6, one of 512 26.7; 190 x 56 x
-// 12 stride 33 with the buffer 103, 65 without 173.
+// Back blur.  Candidates: for each stride of kBackStrides as many tiles as it
+// needs, of equal widths, with the narrowest stride that holds one.  Among those
+// that fit: the fewest rounds of strips per plane, a round of 256 threads
+// counted half; then the widest tile.  The CTA has 256 threads where a pass over
+// a plane has that many strips or fewer and two such CTAs fit an SM, else 512,
+// and the attenuation comes through shared memory where a tile is the whole
+// plane and the buffer fits.  Measured (one subset, us): 64^3 x 8 angles 256
+// threads 14.3, two 32-column tiles of 256 16.3; 96^3 x 12 one tile of 512
+// threads 39.8, two of 256 47.2; 128^3 x 15 one tile of 512 87, two of 256 85;
+// 160^3 x 8 two tiles of 96 columns 117, three of 64 131; 192^3 x 16 x 2 volumes
+// three tiles of 64 columns 338, two of 96 406.  A wider stride than the tile
+// needs takes the second CTA or the attenuation buffer: 132 x 44 x 15 stride 33
+// two CTAs 47.4, 65 one of 256 threads 54.5, one of 512 51.8; 80 x 96 x 12 stride
+// 49 two CTAs 24.9, 65 one of 256 28.6, one of 512 26.7; 190 x 56 x 12 stride 33
+// with the buffer 103, 65 without 173.  Planes of 129 to 192 columns whole, with
+// the buffer, where they had been two tiles of up to 128 (96 angles, us; in
+// brackets with tiles of any width as before the strides were fixed): 57 x 144
+// 308 -> 180 [186], 76 x 160 470 -> 285 [303], 102 x 136 588 -> 424 [426]; two
+// equal tiles of 80 columns in place of 96 or 128: 145 x 136 1219 -> 972.
 BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit)
 {
     BackTiling best{};
     double best_cost = 0.0;
     int last_width = 0;
     const int npad = round_up(n, kStrip), rp = npad / 2, rh = rmax + (rmax & 1);
-    for (int sq : kBackStrides) {
+    for (int widest : kBackStrides) {
         BackTiling t{};
-        t.sq = sq;
-        t.ktpad = std::min(2 * (sq - 1), round_up(nz, kStrip));
-        if (t.ktpad == last_width) break;  // this stride and the wider ones add padding only
+        // as many tiles as this stride needs, of equal widths, with the
+        // narrowest stride that holds one
+        t.ntiles = (nz + 2 * (widest - 1) - 1) / (2 * (widest - 1));
+        t.ktile = t.ntiles == 1 ? nz : round_up((nz + t.ntiles - 1) / t.ntiles, kStrip);
+        t.ktpad = round_up(t.ktile, kStrip);
+        if (t.ktpad == last_width) continue;
         last_width = t.ktpad;
-        t.ktile = std::min(t.ktpad, nz);
-        t.ntiles = (nz + t.ktile - 1) / t.ktile;
+        for (int i = (int)(sizeof kBackStrides / sizeof kBackStrides[0]) - 1; i >= 0; --i)
+            if (2 * (kBackStrides[i] - 1) >= t.ktpad) t.sq = kBackStrides[i];
         t.rh = rh;
         t.npad = npad;
         t.pad_rows = (rmax + 1) / 2;

@@ -76,20 +76,22 @@ def test_planes_that_fit_are_accepted(tilings):
 
 
 def test_back_tilings_carry_no_padding(tilings):
-    """The back blur's stride is the narrowest that holds its tile, a CTA of 256
-    threads is one of two that fit an SM, and a whole plane's attenuation is
-    staged where the buffer fits."""
-    strides = (9, 17, 33, 49, 65)  # kBackStrides
+    """The back blur's stride is the narrowest that holds its tile, its tiles are
+    equal, a CTA of 256 threads is one of two that fit an SM, a plane of up to 192
+    columns is whole and its attenuation staged where that fits."""
+    strides = (9, 17, 33, 49, 65, 81, 97)  # kBackStrides
     shapes = [(n, nz, r, 1) for n in range(32, 193, 3) for nz in range(24, 193, 4) for r in (3, 9, 15, 19)]
     halved = staged = 0
     for (n, nz, r, _), t in zip(shapes, tilings(shapes)):
         assert t["smem"] > 0, (n, nz, r)
-        width = min(s for s in strides if min(2 * (s - 1), _up(nz, 16)) == t["ktpad"])
-        assert t["sq"] == width, (n, nz, r, t)
+        assert t["sq"] == min(s for s in strides if 2 * (s - 1) >= t["ktpad"]), (n, nz, r, t)
+        assert t["ktpad"] == _up(-(-nz // t["ntiles"]), 16), (n, nz, r, t)
         assert t["threads"] in (256, 512)
         if t["threads"] == 256:
             assert 2 * (t["smem"] + 1024) <= 228 * 1024, (n, nz, r, t)
             halved += 1
+        if n <= 80 and nz <= 192 and r <= 9:
+            assert t["ntiles"] == 1, (n, nz, r, t)
         rp, rh = _up(n, 16) // 2, _up(r, 2)
         bare = 16 * (rp * ((t["ktpad"] + 2 * rh) // 2 | 1) + (rp + 2 * ((r + 1) // 2)) * t["sq"]) + 2 * 21 * 4
         fits = t["ntiles"] == 1 and _up(bare, 16) + 4 * n * nz + 8 <= LIMIT
