@@ -299,6 +299,7 @@ uint32_t bf16_tmem_cols(int n, int tiles);  // TMEM columns: `tiles` n-column ac
 int bf16_occupancy(int n);
 
 PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit);
+int depth_chunks(long items, long slots, long most);
 BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit);
 cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t st);
 cudaError_t launch_blur_back(const BlurBackArgs& a, cudaStream_t st);

@@ -97,6 +97,24 @@ PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit)
     return best;  // smem == 0: does not fit
 }
 
+// Depth chunks, at most `most`, of a launch whose every chunk is `items` CTAs,
+// on a device that holds `slots` CTAs at a time: as many as fill one wave, or,
+// where that leaves much of it empty, the fewest whose waves take a sixth less
+// depth.  Two 64-column tiles and 48 angles are 96 CTAs on 152 SMs: in one chunk
+// two volumes are two waves of the whole depth, in three chunks four waves of a
+// third (forward, us): 132 x 128 1609 -> 1084, 160 x 104 2164 -> 1467, 128 x 160
+// 1489 -> 1008, 102 x 188 1101 -> 758.  A launch that fills a wave stays as it is.
+int depth_chunks(long items, long slots, long most)
+{
+    if (items >= slots) return 1;
+    const long first = std::max<long>(1, std::min(most, slots / items));
+    const auto waves = [&](long c) { return (items * c + slots - 1) / slots; };
+    long best = first;
+    for (long c = first + 1; c <= std::min(most, 4 * first); ++c)
+        if (6 * waves(c) * best < 5 * waves(best) * c) best = c;
+    return (int)best;
+}
+
 // Back blur.  Candidates: for each stride of kBackStrides as many tiles as it
 // needs, of equal widths, with the narrowest stride that holds one.  Among those
 // that fit: the fewest rounds of strips per plane, a round of 256 threads

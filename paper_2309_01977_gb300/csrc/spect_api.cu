@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdint>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -272,11 +273,10 @@ void build_psf(const spect_geom& g, int n, bool psf, double offset, std::vector<
 
 // ---------------------------------------------------------------- launches
 
-int chunk_target(const spect_plan* p, long items, int occ)
+// Depth chunks of a launch of `items` CTAs a chunk, at most `cap`.
+int chunk_target(const spect_plan* p, long items, int occ, size_t cap = SIZE_MAX)
 {
-    const long target = (long)p->num_sms * occ;
-    if (items >= target) return 1;
-    return (int)std::max<long>(1, std::min<long>(std::max(1, p->n / 2), target / items));
+    return depth_chunks(items, (long)p->num_sms * occ, (long)std::min<size_t>(cap, std::max(1, p->n / 2)));
 }
 
 // proj (or, with y, the ratio y / (p + s)) = H_sel x.  The depth split
@@ -289,8 +289,8 @@ int run_forward(spect_plan* p, spect_plan_scratch& sc, const float* x, float* ou
 {
     const PlaneTiling& t = p->tiling;
     // never more chunks than the partial buffer holds for one batch entry
-    const int chunks = (int)std::min<size_t>(chunk_target(p, (long)n_sel * (p->bf16 ? 1 : t.ntiles), p->fwd_occ),
-                                             std::max<size_t>(1, p->partial_planes / (size_t)n_sel));
+    const int chunks = chunk_target(p, (long)n_sel * (p->bf16 ? 1 : t.ntiles), p->fwd_occ,
+                                    std::max<size_t>(1, p->partial_planes / (size_t)n_sel));
     // the reduction pass also applies T_fov
     const bool use_partials = chunks > 1 || y != nullptr || p->d_fov != nullptr;
     const size_t vol = vol_elems(p), plane = plane_elems(p);
