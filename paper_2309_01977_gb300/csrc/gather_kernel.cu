@@ -64,11 +64,11 @@ constexpr int kGatherThreads = 64;
 // Angles are taken two at a time so that the table and volume loads of both
 // are in flight together; the sum runs over angles in order, then over each
 // angle's entries in table order, so it is deterministic.  Bound by the chain
-// of loads (few warps: 13 an SM at 64^3): the next pair's entries and the
-// epilogue's operands are on their way during the sums, and CTAs of two warps
-// spread over the SMs in one wave.  64^3 x 8 angles, in an OSEM run: 15.4 ->
-// 12.2 us with the events around it, 16 subiterations 654 -> 577 us.
-__global__ void __launch_bounds__(kGatherThreads, 7) gather_kernel(GatherArgs a)
+// of loads: CTAs of two warps spread over the SMs in one wave.  kBlocks CTAs an
+// SM cap the registers: 8 leave all loads of a pair of angles in flight at once,
+// 16 twice the warps (see launch_gather).
+template <int kBlocks>
+__global__ void __launch_bounds__(kGatherThreads, kBlocks) gather_kernel(GatherArgs a)
 {
     launch_dependents();
     const int n = a.n, nz = a.nz, zw = nz >> 2;
@@ -90,26 +90,18 @@ __global__ void __launch_bounds__(kGatherThreads, 7) gather_kernel(GatherArgs a)
     const float* bb = a.bvol + (size_t)b * a.n_sel * vol + 4 * z4;
     const int2* __restrict__ tab = a.tab;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    // table entries of angles g and g + 1, loaded a pair ahead (an angle past
-    // the end: none)
-    int2 e0[kMaxCand], e1[kMaxCand];
+    // table entries of angle g (past the end: none)
     auto entries = [&](int g, int2 (&e)[kMaxCand]) {
         const bool in = g < a.n_sel;
         const int2* t = tab + ((size_t)a.sel[in ? g : 0] * n * n + col) * kMaxCand;
 #pragma unroll
         for (int q = 0; q < kMaxCand; ++q) e[q] = in ? __ldg(t + q) : make_int2(0, 0);
     };
-    entries(0, e0);
-    entries(1, e1);
     wait_prerequisites();  // up to here plan data only
-    // the image and sensitivity of the epilogue, on their way during the sums
-    const bool upd = a.upd.mode != kUpdNone;
-    const size_t i4 = ((size_t)col * nz >> 2) + z4;
-    float4* o = reinterpret_cast<float4*>(a.out + (size_t)b * vol) + i4;
-    float4 xv = acc, sv = acc;
-    if (upd || a.accumulate) xv = *o;
-    if (upd) sv = reinterpret_cast<const float4*>(a.upd.sens)[i4];
     for (int g = 0; g < a.n_sel; g += 2) {
+        int2 e0[kMaxCand], e1[kMaxCand];
+        entries(g, e0);
+        entries(g + 1, e1);
         float4 v0[kMaxCand], v1[kMaxCand];
         float w0[kMaxCand], w1[kMaxCand];
         const float* b0 = bb + (size_t)g * vol;
@@ -121,8 +113,6 @@ __global__ void __launch_bounds__(kGatherThreads, 7) gather_kernel(GatherArgs a)
             v0[e] = e0[e].y != 0 ? *reinterpret_cast<const float4*>(b0 + e0[e].x) : make_float4(0.f, 0.f, 0.f, 0.f);
             v1[e] = e1[e].y != 0 ? *reinterpret_cast<const float4*>(b1 + e1[e].x) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        entries(g + 2, e0);
-        entries(g + 3, e1);
         auto add = [&](float w, const float4& v) {
             if (w == 0.f) return;
             acc.x = fmaf(w, v.x, acc.x);
@@ -135,6 +125,12 @@ __global__ void __launch_bounds__(kGatherThreads, 7) gather_kernel(GatherArgs a)
 #pragma unroll
         for (int e = 0; e < kMaxCand; ++e) add(w1[e], v1[e]);
     }
+    const bool upd = a.upd.mode != kUpdNone;
+    const size_t i4 = ((size_t)col * nz >> 2) + z4;
+    float4* o = reinterpret_cast<float4*>(a.out + (size_t)b * vol) + i4;
+    float4 xv = make_float4(0.f, 0.f, 0.f, 0.f), sv = xv;
+    if (upd || a.accumulate) xv = *o;
+    if (upd) sv = reinterpret_cast<const float4*>(a.upd.sens)[i4];
     if (upd)
         *o = update4_sv(a.upd, xv, acc, sv, i4);
     else if (a.accumulate)
@@ -152,7 +148,15 @@ cudaError_t launch_gather(const GatherArgs& a, cudaStream_t st)
     else
         warps = ((long)a.n * a.n + (32 / a.lanes_per_col) - 1) / (32 / a.lanes_per_col);
     const long blocks = (warps * 32 + kGatherThreads - 1) / kGatherThreads;
-    return launch_early(gather_kernel, a, dim3((unsigned)blocks, a.batch), kGatherThreads, 0, st);
+    const dim3 grid((unsigned)blocks, a.batch);
+    // 8 CTAs an SM where they hold a volume's warps in one wave, else 16.  12
+    // angles in an OSEM run, us with the events around it, CTAs of 8 warps -> 8 CTAs
+    // an SM / 16 (7 with the next pair's entries ahead): 40 x 36 16.0 -> 10.3 / 13.0
+    // (12.3), 64^3 16.5 -> 13.0 / 14.5 (14.3), 57 x 80 17 -> 18.5 / 17.3 (18.5), 80
+    // x 160 48 -> 53 / 45 (54), 112 x 136 90 -> 96 / 77 (102), 128 x 188 122 -> 131 /
+    // 103 (136).
+    if (warps <= 16L * a.num_sms) return launch_early(gather_kernel<8>, a, grid, kGatherThreads, 0, st);
+    return launch_early(gather_kernel<16>, a, grid, kGatherThreads, 0, st);
 }
 
 }  // namespace spect

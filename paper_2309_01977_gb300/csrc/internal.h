@@ -219,6 +219,7 @@ struct GatherArgs {
     const int* sel;        // [n_sel] angle ids
     int n, nz, n_sel, batch;
     int lanes_per_col;     // 32, or the power of two >= nz/4 when nz/4 < 32
+    int num_sms;
     float* out;            // [batch][n][n][nz]
     int accumulate;        // add into out instead of overwriting
     UpdateSpec upd;        // mode != kUpdNone: update x (`out`) with the finished back projection

@@ -493,6 +493,7 @@ int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_
                 while (l < p->nz / 4 && l < 32) l <<= 1;
                 ga.lanes_per_col = l;
             }
+            ga.num_sms = p->num_sms;
             ga.out = out_b;
             ga.accumulate = g0 > 0 || accumulate;
             if (fused) ga.upd = *upd;
