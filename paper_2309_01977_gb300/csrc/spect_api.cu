@@ -273,6 +273,42 @@ void build_psf(const spect_geom& g, int n, bool psf, double offset, std::vector<
 
 // ---------------------------------------------------------------- launches
 
+// z segment of the tiled gather: whole columns up to 128 long (each run of
+// footprint rows is one contiguous copy), longer ones in equal segments of 80 to
+// 128 where there are such, else 0.
+int gather_segment(int nz)
+{
+    if (nz <= 128) return nz;
+    for (int d = 2; nz / d >= 80; ++d)
+        if (nz % (4 * d) == 0 && nz / d <= 128) return nz / d;
+    return 0;
+}
+
+// Whether a plan's gather is tiled, by CTAs of a tile and z segment each.  A
+// segment's length hardly changes the time of a CTA, of which two fit an SM; the
+// per-column gather's time goes with the voxels, and up to 64 along z its warps
+// take two columns, up to 32 four.  So, with tiled / per column of 12 angles in an
+// OSEM run, us with the events around it:
+//   65 to 128 along z: from 96^2 planes on (96 x 80 27 / 36, 102 x 96 35 / 40, 128
+//   x 128 38 / 59), and where pairs of CTAs share a tile's angles (run_back) from
+//   88^2 on with 8 angles or more (88 x 88 x 8 angles 22 / 22, x 12 26 / 30, 92 x
+//   96 x 16 31 / 42; 80 x 96 x 8 22 / 20);
+//   33 to 64: only where the tiles are one full wave (128 x 64 36 / 33, its back
+//   projection of 48 angles and two volumes 233 / 246; 132 x 48 36 / 34 and 233 /
+//   254; 96 x 64 27 / 22, 112 x 48 35 / 28, 124 x 64 35 / 31, 144 x 64 60 / 43);
+//   32 and less: never (96 x 24 32 / 16, 128 x 24 35 / 20, 160 x 24 63 / 30);
+//   segments: not where the second wave would be less than half full (96 x 160
+//   53 / 61, 102 x 160 81 / 68, 112 x 160 98 / 80, 128 x 160 101 / 100, 160^3 148 /
+//   150, its back projection of 48 angles and two volumes 1041 / 1121).
+bool gather_by_tiles(const spect_plan* p, int zs)
+{
+    if (zs == 0 || p->nz <= 32) return false;
+    const int side = (p->n + kGtT - 1) / kGtT, ctas = side * side * (p->nz / zs);
+    if (p->nz <= 64) return p->n >= 128 && ctas <= 2 * p->num_sms;
+    if (p->nz > zs) return p->n >= 96 && (ctas <= 2 * p->num_sms || ctas >= 3 * p->num_sms);
+    return p->n >= 96 || (p->n >= 88 && ctas <= p->num_sms && p->max_subset >= 8);
+}
+
 // Depth chunks of a launch of `items` CTAs a chunk, at most `cap`.
 int chunk_target(const spect_plan* p, long items, int occ, size_t cap = SIZE_MAX)
 {
@@ -463,13 +499,15 @@ int run_back(spect_plan* p, spect_plan_scratch& sc, const float* proj, float* x_
                 gt.zs = p->gt_zs;
                 gt.rows_cap = p->gt_rows;
                 gt.stages = p->gt_stages;
-                // Fewer tiles than SMs: pairs of CTAs that share the angles.  96^3 x
-                // 12 angles, one subset in an OSEM run, us: 34.1 -> 27.4 with the
-                // events around it; a subset's sensitivity 28.4 -> 22.4; back of 96
-                // angles 479 -> 407.  With as many tiles as SMs or more it costs
-                // a second wave: 112^3 36.6 -> 48.6, 128^3 43.6 -> 57.7.  Blind to
-                // the batch, so that a volume is summed in the same order alone and
-                // in a batch (two volumes at 96^3 739 -> 785, three 1078 -> 1073).
+                // Fewer tiles than SMs (planes of 88^2 to 96^2): pairs of CTAs that
+                // share the angles.  96^3 x 12 angles, one subset in an OSEM run,
+                // us: 34.1 -> 27.4 with the events around it; 88^3 32.8 -> 26.9; a
+                // subset's sensitivity 28.4 -> 22.4; back of 96 angles 479 -> 407.
+                // With as many tiles as SMs or more it costs a second wave: 112^3
+                // 36.6 -> 48.6, 128^3 43.6 -> 57.7.  Blind to the batch, so that a
+                // volume is summed in the same order alone and in a batch (two
+                // volumes at 96^3 739 -> 785, three 1078 -> 1073; two at 88^3 x 12
+                // angles 126 -> 109 with the back blur).
                 gt.pair = ng >= 4 && p->gt_tiles * (p->nz / p->gt_zs) <= p->num_sms &&
                           gather_pair_fits(p->gt_rows, p->gt_zs, p->gt_stages);
                 gt.out = out_b;
@@ -1006,20 +1044,11 @@ int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream,
     }
     SPECT_CK(cudaMemcpyAsync(p->d_rad, radw.data(), radw.size() * sizeof(int), cudaMemcpyHostToDevice, st), "copy radii");
     SPECT_CK(cudaMemcpyAsync(p->d_sel_all, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, st), "copy angles");
-    // Gather tables.  Tiled (footprints staged in shared memory) for planes
-    // of at least 96 x 96: 8 x 8 tiles, whole columns up to 128 long (each run
-    // of footprint rows is one contiguous copy), longer ones in equal segments
-    // of 80 to 128 where there are such, and two footprint buffers (one angle
-    // in flight; a third buffer measured slower on GB300).  Else the
-    // per-column gather.  Tiled against per column, one subset with the events
-    // around it, us: 64^3 x 8 angles 21.6 / 12.2, 80 x 80 x 64 x 8 22.5 / 22.5
-    // (a whole iteration 487 / 466), 96^3 x 12 27.4 (pairs) / 39.4, 112 x 112 x
-    // 96 x 12 36.6 / 58.2; launches alone: 160^3 x 8 (two segments of 80) 89 /
-    // 121, 192^3 x 16 (two of 96) 222 / 313, in three of 64 318.
-    int zs = p->nz <= 128 ? p->nz : 0;
-    for (int d = 2; zs == 0 && p->nz / d >= 80; ++d)
-        if (p->nz % (4 * d) == 0 && p->nz / d <= 128) zs = p->nz / d;
-    p->gather_tiled = p->n >= 96 && zs > 0;
+    // Gather tables: tiled (footprints staged in shared memory; two footprint
+    // buffers, one angle in flight: a third buffer measured slower on GB300) or
+    // per column.
+    const int zs = gather_segment(p->nz);
+    p->gather_tiled = gather_by_tiles(p, zs);
     if (p->gather_tiled) {
         p->gt_T = kGtT;
         const int tx = (p->n + p->gt_T - 1) / p->gt_T;
