@@ -45,9 +45,10 @@
  * Memory: every pointer argument is a device pointer (the caller owns it) to
  * contiguous FP32 data, LOR arrays 8-byte aligned, images 16-byte aligned;
  * diag_out is a host pointer.  The plan owns its taps, a copy of mu, its
- * scratch images and, from the first call with at least one line per 32
- * voxels on, the image's quads (pet_forward, pet_lm_osem_run) and the back
- * projection's (pet_back, pet_lm_osem_run): 16 bytes a cell of nx x ny x nz
+ * scratch images and, from the first call with many lines on (at least one per
+ * 32 voxels; back projections and calls with time of flight at least some 50,000
+ * to 500,000 on top, by grid), the image's quads (pet_forward, pet_lm_osem_run)
+ * and the back projection's (pet_back, pet_lm_osem_run): 16 bytes a cell of nx x ny x nz
  * cells each (axes rounded up to the walk's bricks; 104 MB at 204 x 204 x 154).
  * That first call allocates them, which may wait for the device, under stream
  * capture as well, if they take half of the free memory at most; where it

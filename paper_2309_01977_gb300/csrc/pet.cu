@@ -1044,17 +1044,44 @@ bool take_quads(pet_plan* p, bool image, bool back, size_t bytes)
     return true;
 }
 
-// Whether a call walks quads: at least one line per 32 voxels (building,
-// clearing and folding quads moves about 100 bytes a voxel and axis, some 0.1
-// ms at 204 x 204 x 154, which a line's saving of about 1 ns repays from 0.1 M
-// lines, 1 / 64 of the voxels, on), lattices that 32-bit indexes reach, and the
-// memory for the sets that the mode needs, kept by the plan.  Where there is
-// none the image is walked, and a later call tries again.
+// Whether `lines` lines pay for the quads: at least one per 32 voxels (building,
+// clearing and folding quads moves about 100 bytes a voxel and axis), and with
+// less than a wave of the image walk, which then takes the time of one line, as
+// many as the mode needs.  Events of the head phantom, us, image walk / quads:
+//   forward                 64 x 64 x 40, 8192 lines 104 / 87; 96 x 96 x 64, 24576
+//                           143 / 110; 204 x 204 x 154, 262144 610 / 430
+//   back                    64^3, 16384 68 / 88, 49152 100 / 100, 131072 172 / 154;
+//                           128 x 128 x 90, 49152 155 / 139
+//   OSEM                    64^3, 8192 161 / 146; 128 x 128 x 90, 49152 330 / 247
+//   with time of flight:
+//   forward                 64 x 64 x 120, 65536 119 / 136, 131072 210 / 187; 96 x 96
+//                           x 64, 24576 136 / 124
+//   back                    64^3, 131072 159 / 187, 524288 386 / 388; 64 x 64 x 120,
+//                           131072 194 / 192; 128 x 128 x 90, 98304 201 / 206, 131072
+//                           247 / 232
+//   OSEM                    64^3, 65536 174 / 197, 98304 211 / 230, 131072 304 / 249;
+//                           204 x 204 x 154, 98304 580 / 614, 262144 1240 / 864
+constexpr long long kImageWave = 152 * 3 * kPetThreads;  // with time of flight 3 CTAs an SM
+
 template <int kMode>
-bool use_quads(pet_plan* p, long long lines)
+bool quads_pay(const pet_plan* p, long long lines, bool tof)
+{
+    if (lines < p->voxels / 32) return false;
+    if (!tof) return kMode != kModeBack || lines >= 3 << 14;
+    const bool waves = lines > kImageWave;
+    if (kMode == kModeFwd) return waves || p->voxels >= 1 << 19;
+    if (kMode == kModeBack) return waves && (p->voxels >= 3 << 17 || lines >= 1 << 19);
+    return waves;
+}
+
+// Whether a call walks quads: where that pays, on lattices that 32-bit indexes
+// reach, with the memory for the sets that the mode needs, kept by the plan.
+// Where there is none the image is walked, and a later call tries again.
+template <int kMode>
+bool use_quads(pet_plan* p, long long lines, bool tof)
 {
     const long long cells = std::max(quad_cells(p->grid, 0), quad_cells(p->grid, 1));
-    if (lines < p->voxels / 32 || cells >= (1ll << 31) - (1ll << 23) || p->voxels >= (1ll << 31)) return false;
+    if (!quads_pay<kMode>(p, lines, tof) || cells >= (1ll << 31) - (1ll << 23) || p->voxels >= (1ll << 31)) return false;
     return take_quads(p, kMode != kModeBack, kMode != kModeFwd, (size_t)cells * sizeof(float4));
 }
 
@@ -1080,7 +1107,7 @@ void launch_quad_axis(pet_plan* p, const LmArgs& a, cudaStream_t st)
 template <int kMode>
 int launch_walk(pet_plan* p, const char* name, LmArgs a, cudaStream_t st)
 {
-    const bool quads = use_quads<kMode>(p, a.count);
+    const bool quads = use_quads<kMode>(p, a.count, a.tof_bin != nullptr);
     const int kernels = !quads ? 1 : kMode == kModeEm ? 7 : 5;
     return launch(p, name, st, kernels, [&] {
         if (quads) {

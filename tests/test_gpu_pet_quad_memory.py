@@ -46,20 +46,28 @@ def _free():
 VOXELS = 64 ** 3
 
 
-@pytest.mark.parametrize("lines,quads", [(VOXELS // 32, True), (VOXELS // 32 - 1, False)])
-def test_launches_tell_the_walks_apart(spect_lib, cuda, lines, quads):
+MANY = 3 << 14  # lines from which a back projection without time of flight walks quads
+
+
+@pytest.mark.parametrize("lines,back", [(MANY, 5), (MANY - 1, 1), (VOXELS // 32, 1)])
+def test_launches_tell_the_walks_apart(spect_lib, cuda, lines, back):
     x, lors, q = _inputs(lines)
     plan = _plan()
     one = torch.ones_like(x)
-    assert _launches(spect_lib, lambda: plan.forward(x, lors)) == (5 if quads else 1)
-    assert _launches(spect_lib, lambda: plan.back(q, lors)) == (5 if quads else 1)
-    assert _launches(spect_lib, lambda: plan.lm_osem(lors, q, None, one, x, 0, 1)) == (8 if quads else 2)
+    assert _launches(spect_lib, lambda: plan.forward(x, lors)) == 5
+    assert _launches(spect_lib, lambda: plan.back(q, lors)) == back
+    assert _launches(spect_lib, lambda: plan.lm_osem(lors, q, None, one, x, 0, 1)) == 8
+    few = VOXELS // 32 - 1
+    lors, q = lors[:few].contiguous(), q[:few].contiguous()
+    assert _launches(spect_lib, lambda: plan.forward(x, lors)) == 1
+    assert _launches(spect_lib, lambda: plan.back(q, lors)) == 1
+    assert _launches(spect_lib, lambda: plan.lm_osem(lors, q, None, one, x, 0, 1)) == 2
     plan.close()
 
 
 @pytest.mark.parametrize("call", ["forward", "back"])
 def test_a_projector_takes_its_own_set(spect_lib, cuda, call):
-    x, lors, q = _inputs(VOXELS // 32)
+    x, lors, q = _inputs(MANY)
     warm = _plan()  # the kernels of both walks are loaded
     out = {"forward": torch.empty_like(q), "back": torch.empty_like(x)}
     run = lambda p: p.forward(x, lors, out=out[call]) if call == "forward" else p.back(q, lors, out=out[call])
