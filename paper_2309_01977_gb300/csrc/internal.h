@@ -300,6 +300,7 @@ uint32_t bf16_tmem_cols(int n, int tiles);  // TMEM columns: `tiles` n-column ac
 int bf16_occupancy(int n);
 
 PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit);
+PlaneTiling many_tiling(const PlaneTiling& t);
 int depth_chunks(long items, long slots, long most);
 BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit);
 cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t st);
@@ -342,12 +343,16 @@ cudaError_t launch_prior_grad(const float* x, float* grad, int n, int nz, int pr
 void spect_internal_set_error(const char* msg);
 // Adds kernels launched outside spect_api.cu to spect_kernel_launches().
 void spect_internal_count_launches(unsigned long long kernels);
+// spect_plan_create; osem_only: without the partial planes of plain projections in
+// small CTAs (a server's slots, whose memory is reserved without them).
+int spect_internal_plan_create(const spect_geom* geom, const float* mu_dev, void* stream, spect_plan** out,
+                               bool osem_only);
 
 // Scratch of the calls queued on one stream of a plan: calls on different
 // streams never share it, so they may run concurrently.
 struct spect_plan_scratch {
     cudaStream_t stream = nullptr;
-    float* partials = nullptr;    // forward depth-chunk partials [partial_planes][n][nz]
+    float* partials = nullptr;    // forward depth-chunk partials [max(partial_planes, many_planes)][n][nz]
     float* bvol = nullptr;        // back-projection rotated-frame volumes [bvol_cap][vol]
     float* ratio = nullptr;       // [max_subset][n][nz]
     float* bp = nullptr;          // one volume: back projection of large subsets, other peaks
@@ -368,6 +373,9 @@ struct spect_plan {
     int psf_tables = 1;                     // PSF tables: n_angles for a non-circular orbit, else 1
     int max_subset = 0;
     spect::PlaneTiling tiling{};
+    spect::PlaneTiling many{};      // of the forward in small CTAs (many_occ > 0: a launch may take it)
+    int many_occ = 0;
+    size_t many_planes = 0;         // partial planes that it may write
     spect::BackTiling back{};
     int fwd_occ = 1, back_occ = 1;  // resident forward / back blur CTAs per SM
 
@@ -380,7 +388,7 @@ struct spect_plan {
     std::vector<int*> d_sel;                  // per subset
     float* d_atten = nullptr;                 // [na][vol]
     float* d_sens = nullptr;                  // [M][vol]
-    size_t partial_planes = 0;                // capacity of a scratch's depth-chunk partials, planes
+    size_t partial_planes = 0;                // depth-chunk partials that a launch of `tiling` may write, planes
     int2* d_gtab = nullptr;                   // adjoint-rotation gather tables: [na][n*n][kMaxCand], or
                                               // tiled [na][gt_tiles] strip tables of kGtSliceBytes
     int* d_gdesc = nullptr;                   // tiled gather footprints [na][gt_tiles][kFpDescInts]

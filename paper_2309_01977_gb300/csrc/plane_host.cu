@@ -97,6 +97,23 @@ PlaneTiling plane_tiling(int n, int nz, int rmax, size_t cap, size_t limit)
     return best;  // smem == 0: does not fit
 }
 
+// The forward's tiling in CTAs of a thread per blur strip (64 at least), several
+// to an SM.  A CTA of 256 keeps most of its threads idle in the blur of a short
+// plane, which suits a launch of one or two planes a CTA (their staging takes all
+// threads); a launch of more is bound by the blurs' throughput.  Taken where four or
+// more fit an SM.  Whole projections, us with their reduction, CTAs of that size
+// always -> 256 threads -> by launch: 48 x 24, 96 angles 53 -> 67 -> 51, four
+// volumes 167 -> 220 -> 161; 64^2 x 24, 48 angles, four volumes 156 -> 185 -> 154; 76
+// x 36 the same 230 -> 250 -> 223; with three to an SM (76 x 48) 255 -> 252 -> 260.
+// smem 0 where CTAs would not get smaller.
+PlaneTiling many_tiling(const PlaneTiling& t)
+{
+    PlaneTiling m = t;
+    m.threads = std::max(64, round_up((t.ktpad / 2) * (t.npad / kStrip), 32));
+    if (t.ipt > 1 || m.threads >= t.threads) m.smem = 0;
+    return m;
+}
+
 // Depth chunks, at most `most`, of a launch whose every chunk is `items` CTAs,
 // on a device that holds `slots` CTAs at a time: as many as fill one wave, or,
 // where that leaves much of it empty, the fewest whose waves take a sixth less

@@ -225,7 +225,7 @@ int create_slot(spect_server* sv, Request* r, cudaStream_t st, Slot** out)
     g.det_offsets = sl->offsets.empty() ? nullptr : sl->offsets.data();
     g.det_shifts = sl->shifts.empty() ? nullptr : sl->shifts.data();
     g.fov_mask = sl->fov.empty() ? nullptr : sl->fov.data();
-    int rc = spect_plan_create(&g, (g.flags & SPECT_FLAG_ATTEN) ? sl->d_mu : nullptr, st, &sl->plan);
+    int rc = spect_internal_plan_create(&g, (g.flags & SPECT_FLAG_ATTEN) ? sl->d_mu : nullptr, st, &sl->plan, true);
     if (rc) {
         destroy_slot(sl);
         return rc;

@@ -323,16 +323,26 @@ int run_forward(spect_plan* p, spect_plan_scratch& sc, const float* x, float* ou
                 int batch, const float* y, float s, double* diag_blocks, int* n_diag, cudaStream_t st,
                 const float* s_ptr = nullptr, float scale = 1.f)
 {
-    const PlaneTiling& t = p->tiling;
     // never more chunks than the partial buffer holds for one batch entry
-    const int chunks = chunk_target(p, (long)n_sel * (p->bf16 ? 1 : t.ntiles), p->fwd_occ,
-                                    std::max<size_t>(1, p->partial_planes / (size_t)n_sel));
+    const long items = (long)n_sel * (p->bf16 ? 1 : p->tiling.ntiles);
+    size_t planes = p->partial_planes;
+    int chunks = chunk_target(p, items, p->fwd_occ, std::max<size_t>(1, planes / (size_t)n_sel));
+    // Small CTAs (many_tiling) for a projection whose CTAs would have five planes
+    // of depth or more, or whose batch makes several waves of them; the latter
+    // keep the chunks, so that a volume has the same bits alone and in a batch.
+    const bool deep = p->n >= 5 * chunks;
+    const bool many = !y && p->many_occ > 0 && (deep || batch * items * chunks > 2L * p->num_sms * p->fwd_occ);
+    if (many) {
+        planes = p->many_planes;
+        if (deep) chunks = chunk_target(p, items, p->many_occ, std::max<size_t>(1, planes / (size_t)n_sel));
+    }
+    const PlaneTiling& t = many ? p->many : p->tiling;
     // the reduction pass also applies T_fov
     const bool use_partials = chunks > 1 || y != nullptr || p->d_fov != nullptr;
     const size_t vol = vol_elems(p), plane = plane_elems(p);
     int bper = batch;
     if (use_partials)
-        bper = (int)std::max<size_t>(1, std::min<size_t>(batch, p->partial_planes / ((size_t)n_sel * chunks)));
+        bper = (int)std::max<size_t>(1, std::min<size_t>(batch, planes / ((size_t)n_sel * chunks)));
     if (n_diag) *n_diag = 0;
     for (int b0 = 0; b0 < batch; b0 += bper) {
         const int nb = std::min(bper, batch - b0);
@@ -577,7 +587,7 @@ int scratch_for(spect_plan* p, cudaStream_t st, spect_plan_scratch** out)
     s->stream = st;
     const size_t vol = vol_elems(p), plane = plane_elems(p);
     int rc;
-    if ((rc = dev_alloc(p, &s->partials, p->partial_planes * plane)) ||
+    if ((rc = dev_alloc(p, &s->partials, std::max(p->partial_planes, p->many_planes) * plane)) ||
         (rc = dev_alloc(p, &s->bvol, p->bvol_cap * vol)) ||
         (rc = dev_alloc(p, &s->ratio, (size_t)p->max_subset * plane)) ||
         (rc = dev_alloc(p, &s->bp, vol)) ||
@@ -847,6 +857,14 @@ const char* spect_status_str(int status)
 
 int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream, spect_plan** out)
 {
+    return spect_internal_plan_create(geom, mu_dev, stream, out, false);
+}
+
+}  // extern "C"
+
+int spect_internal_plan_create(const spect_geom* geom, const float* mu_dev, void* stream, spect_plan** out,
+                               bool osem_only)
+{
     CallRange range("spect_plan_create");
     if (!out) return fail(SPECT_EINVAL, "out is NULL");
     *out = nullptr;
@@ -971,6 +989,14 @@ int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream,
     const size_t target = (size_t)p->num_sms * p->fwd_occ;
     // at most four planes per SM: what a server reserves for a slot
     p->partial_planes = std::max<size_t>(std::min<size_t>(2 * target, 4 * (size_t)p->num_sms), (size_t)p->max_subset);
+    if (!p->bf16 && !osem_only) {
+        p->many = many_tiling(p->tiling);
+        p->many_occ = p->many.smem ? forward_max_blocks_per_sm(p->many) : 0;
+        if (p->many_occ < 4) p->many_occ = 0;
+        p->many.ctas = p->many_occ;
+        if (p->many_occ)
+            p->many_planes = std::max<size_t>((size_t)std::min(2 * p->many_occ, 16) * p->num_sms, p->partial_planes);
+    }
     p->bvol_cap = (size_t)std::max(p->max_subset, 16);
     if ((rc = dev_alloc(p, &p->d_cs, p->na)) ||
         (rc = dev_alloc(p, &p->d_taps, taps.size())) ||
@@ -1105,6 +1131,8 @@ int spect_plan_create(const spect_geom* geom, const float* mu_dev, void* stream,
     *out = p;
     return SPECT_OK;
 }
+
+extern "C" {
 
 int spect_plan_destroy(spect_plan* plan)
 {
@@ -1321,7 +1349,7 @@ int spect_plan_release_stream(spect_plan* plan, void* stream)
         cudaError_t e = cudaStreamSynchronize(st);  // its last use has finished
         if (e != cudaSuccess) return cuda_fail(e, "synchronize the released stream");
         const size_t vol = vol_elems(plan), plane = plane_elems(plan);
-        dev_free(plan, s->partials, plan->partial_planes * plane * sizeof(float));
+        dev_free(plan, s->partials, std::max(plan->partial_planes, plan->many_planes) * plane * sizeof(float));
         dev_free(plan, s->bvol, plan->bvol_cap * vol * sizeof(float));
         dev_free(plan, s->ratio, (size_t)plan->max_subset * plane * sizeof(float));
         dev_free(plan, s->bp, vol * sizeof(float));
