@@ -443,26 +443,31 @@ cudaError_t launch_wsum(float* out, const float* const* in, const float* w, int 
 //   a pair whose RDP denominator is 0 contributing 0.
 // So does a pair whose S (below) is subnormal: 1 / S is past the largest float
 // there, and two equal neighbours would give 0 inf.
-// A thread walks kPriorRun voxels along i, z fastest over the lanes, with the
-// 27 values around its voxel in registers (nine loads a voxel).  Bound by the
-// RDP's arithmetic, 26 terms a voxel: with S the denominator's root, a term is
+// A thread a voxel, z fastest, the planes' columns (j, k) in one index, so that no
+// thread is idle whatever the shape and one index is divided.  Bound by the RDP's
+// arithmetic, 26 terms a voxel: with S the denominator's root, a term is
 // (d / S) ((S + 2 b) / S), one reciprocal in place of a division by S^2 (which
-// also underflowed for S below 1e-19), and no index is divided.
-// 128^3, relative difference: 89 -> 72 us a launch.
-constexpr int kPriorRun = 4, kPriorZ = 32, kPriorJ = 8;
+// also underflowed for S below 1e-19).  Relative difference in a BSREM run, us with
+// the events around it, divisions and three divided indexes -> runs of four voxels
+// in blocks of 32 x 8 -> this: 128^3 82 -> 83 -> 75, 106 x 100 48 -> 66 -> 50, 64^3 17
+// -> 21 -> 16, 40 x 36 11 -> 20 -> 10, 90 x 72 29 -> 44 -> 29.
+constexpr int kPriorThreads = 256;
 
 template <bool kRdp>
-__global__ void __launch_bounds__(kPriorZ * kPriorJ) prior_grad_kernel(const float* __restrict__ x,
-                                                                       float* __restrict__ grad, int n, int nz,
-                                                                       float delta, float gamma)
+__global__ void __launch_bounds__(kPriorThreads) prior_grad_kernel(const float* __restrict__ x,
+                                                                   float* __restrict__ grad, int n, int nz,
+                                                                   float delta, float gamma)
 {
-    const int k = blockIdx.x * kPriorZ + threadIdx.x, j = blockIdx.y * kPriorJ + threadIdx.y;
-    if (k >= nz || j >= n) return;
-    const int i0 = blockIdx.z * kPriorRun;
+    const size_t plane = (size_t)n * nz;
+    const unsigned per = (unsigned)((plane + kPriorThreads - 1) / kPriorThreads);  // blocks a plane
+    const int i = blockIdx.x / per;
+    const size_t col = (size_t)(blockIdx.x - i * per) * kPriorThreads + threadIdx.x;
+    if (col >= plane) return;
+    const int j = plane >> 31 ? (int)(col / nz) : (int)col / nz, k = (int)(col - (size_t)j * nz);
     const float inv2d2 = 1.f / (2.f * delta * delta);
     const float wt[4] = {0.f, 2.f, 2.f / sqrtf(2.f), 2.f / sqrtf(3.f)};
     // columns (j + dj, k + dk): inside the volume, and their offsets (this
-    // voxel's own outside)
+    // voxel's own outside); planes i - 1 and i + 1 alike
     bool in[9];
     int off[9];
 #pragma unroll
@@ -471,60 +476,45 @@ __global__ void __launch_bounds__(kPriorZ * kPriorJ) prior_grad_kernel(const flo
         in[c] = j + dj >= 0 && j + dj < n && k + dk >= 0 && k + dk < nz;
         off[c] = in[c] ? dj * nz + dk : 0;
     }
-    const size_t plane = (size_t)n * nz;
-    const float* col = x + (size_t)j * nz + k;
-    float v[3][9];  // planes i - 1, i, i + 1
-    auto load = [&](int i, float (&p)[9]) {
-        const float* q = col + (size_t)min(max(i, 0), n - 1) * plane;
+    float v[3][9];
 #pragma unroll
-        for (int c = 0; c < 9; ++c) p[c] = __ldg(q + off[c]);
-    };
-    load(i0 - 1, v[0]);
-    load(i0, v[1]);
+    for (int p = 0; p < 3; ++p) {
+        const float* q = x + (size_t)min(max(i + p - 1, 0), n - 1) * plane + col;
 #pragma unroll
-    for (int r = 0; r < kPriorRun; ++r) {
-        const int i = i0 + r;
-        if (i >= n) break;
-        load(i + 1, v[2]);
-        const float a = v[1][4];
-        float g = 0.f;
+        for (int c = 0; c < 9; ++c) v[p][c] = __ldg(q + off[c]);
+    }
+    const float a = v[1][4];
+    float g = 0.f;
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            const bool plane_in = p == 1 || (p == 0 ? i > 0 : i + 1 < n);
-#pragma unroll
-            for (int c = 0; c < 9; ++c) {
-                if (p == 1 && c == 4) continue;
-                const float w = wt[(p != 1) + (c / 3 != 1) + (c % 3 != 1)];
-                const float b = v[p][c], d = a - b;
-                float t = d * inv2d2;
-                bool ok = plane_in && in[c];
-                if (kRdp) {
-                    const float S = fmaf(gamma, fabsf(d), a + b), q = __frcp_rn(S);
-                    t = (d * q) * (fmaf(2.f, b, S) * q);
-                    ok = ok && !(fabsf(S) < FLT_MIN);
-                }
-                g = fmaf(w, ok ? t : 0.f, g);
-            }
-        }
-        grad[(size_t)i * plane + (size_t)j * nz + k] = g;
+    for (int p = 0; p < 3; ++p) {
+        const bool plane_in = p == 1 || (p == 0 ? i > 0 : i + 1 < n);
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
-            v[0][c] = v[1][c];
-            v[1][c] = v[2][c];
+            if (p == 1 && c == 4) continue;
+            const float w = wt[(p != 1) + (c / 3 != 1) + (c % 3 != 1)];
+            const float b = v[p][c], d = a - b;
+            float t = d * inv2d2;
+            bool ok = plane_in && in[c];
+            if (kRdp) {
+                const float S = fmaf(gamma, fabsf(d), a + b), q = __frcp_rn(S);
+                t = (d * q) * (fmaf(2.f, b, S) * q);
+                ok = ok && !(fabsf(S) < FLT_MIN);
+            }
+            g = fmaf(w, ok ? t : 0.f, g);
         }
     }
+    grad[(size_t)i * plane + col] = g;
 }
 
 cudaError_t launch_prior_grad(const float* x, float* grad, int n, int nz, int prior, float delta, float gamma,
                               cudaStream_t st)
 {
     if ((size_t)n * n * nz == 0) return cudaSuccess;
-    const dim3 block(kPriorZ, kPriorJ);
-    const dim3 grid((nz + kPriorZ - 1) / kPriorZ, (n + kPriorJ - 1) / kPriorJ, (n + kPriorRun - 1) / kPriorRun);
+    const unsigned grid = (unsigned)(((size_t)n * nz + kPriorThreads - 1) / kPriorThreads * n);
     if (prior == SPECT_PRIOR_QUADRATIC)
-        prior_grad_kernel<false><<<grid, block, 0, st>>>(x, grad, n, nz, delta, gamma);
+        prior_grad_kernel<false><<<grid, kPriorThreads, 0, st>>>(x, grad, n, nz, delta, gamma);
     else
-        prior_grad_kernel<true><<<grid, block, 0, st>>>(x, grad, n, nz, delta, gamma);
+        prior_grad_kernel<true><<<grid, kPriorThreads, 0, st>>>(x, grad, n, nz, delta, gamma);
     return cudaGetLastError();
 }
 
