@@ -573,14 +573,15 @@ def run_pet_leg(torch, dev, timed, max_over_ranks, world, k, cpu_seconds: float,
     if os.path.exists(l2):
         with open(l2) as fh:
             prof_l2 = json.load(fh).get(em_name)
-        # the walk gathers from and scatters into quads of the image through
-        # L2: its throughput as a fraction of L2 peak, measured by ncu
+        # the walk waits for the quads that miss L2: HBM traffic as a fraction
+        # of the measured copy bandwidth, with L2 and issue beside it
         if prof_l2:
-            leg["roofline"] = {"bound": "l2", "kernel": em_name, "frac": prof_l2["lts_throughput_frac"],
+            leg["roofline"] = {"bound": "hbm", "kernel": em_name, "frac": prof_l2["hbm_frac"],
+                               "l2_throughput_frac": prof_l2["lts_throughput_frac"],
                                "issue_active_frac": prof_l2["issue_active_frac"], "measured_in_run": False,
-                               "source": "stored: ncu of the same kernel at 3 M prompts, read from "
-                                         "profiles/l2_petlm204.json (profiles/pet_lm_em_petlm204.md); "
-                                         "stale if the kernel has changed since"}
+                               "source": "stored: ncu of the same kernel's walks at 3 M prompts (this run has %d), read "
+                                         "from profiles/l2_petlm204.json (profiles/pet_lm_em_petlm204.md); "
+                                         "stale if the kernel has changed since" % n_ev}
     if with_cpu:
         leg["cpu_baseline"] = pet_cpu_baseline(wl, act, mu, lors, mult, s, sens, cpu_seconds, tof_bin)
     plan.close()

@@ -385,15 +385,15 @@ __global__ void __launch_bounds__(kPetThreads) pet_lm_kernel(LmArgs a)
 // 128-byte bricks of 4 planes x 2 u x 1 w, so that the four share about two
 // lines (along the axis a line moves by half a cell in u and less in w).  What
 // bounds it now is the latency of misses past L2: at 204 x 204 x 154 the two sets
-// of quads are 104 MB each, 43 % of the sectors hit, and HBM moves 3.8 TB/s; L1
+// of quads are 104 MB each, 43 % of the sectors hit, and HBM moves 3.6 TB/s; L1
 // and the issue slots are half busy.
 // Measured, image walk -> quads in plane order -> bricks: an iteration of 3 M
 // events in 3 subsets at 204 x 204 x 154 with time of flight 9.7 -> 6.95 ->
 // 5.58 ms; 128 x 128 x 90, 1 M lines without, forward and back 2.60 -> 1.46 ->
-// 1.23 ms.  64 registers (32 warps an SM) are worth more than a wider batch:
-// 2.79 -> 2.20 ms a subset.  Tried and not better: gathering and scattering in
-// separate launches (2.71 ms), the time-of-flight lines slab by slab along the
-// axis (2.27 ms).
+// 1.23 ms.  64 registers (32 warps an SM at most, 28 on average) are worth more
+// than a wider batch: 2.79 -> 2.20 ms a subset.  Tried and not better: gathering
+// and scattering in separate launches (2.71 ms), the time-of-flight lines slab by
+// slab along the axis (2.27 ms).
 
 constexpr int kQuadThreads = 128;
 

@@ -141,16 +141,17 @@ int depth_chunks(long items, long slots, long most)
 // plane and the buffer fits.  Measured (one subset, us): 64^3 x 8 angles 256
 // threads 14.3, two 32-column tiles of 256 16.3; 96^3 x 12 one tile of 512
 // threads 39.8, two of 256 47.2; 128^3 x 15 one tile of 512 87, two of 256 85;
-// 160^3 x 8 two tiles of 96 columns 117, three of 64 131; 192^3 x 16 x 2 volumes
-// three tiles of 64 columns 338, two of 96 406.  A wider stride than the tile
-// needs takes the second CTA or the attenuation buffer: 132 x 44 x 15 stride 33
-// two CTAs 47.4, 65 one of 256 threads 54.5, one of 512 51.8; 80 x 96 x 12 stride
-// 49 two CTAs 24.9, 65 one of 256 28.6, one of 512 26.7; 190 x 56 x 12 stride 33
-// with the buffer 103, 65 without 173.  Planes of 129 to 192 columns whole, with
-// the buffer, where they had been two tiles of up to 128 (96 angles, us; in
-// brackets with tiles of any width as before the strides were fixed): 57 x 144
-// 308 -> 180 [186], 76 x 160 470 -> 285 [303], 102 x 136 588 -> 424 [426]; two
-// equal tiles of 80 columns in place of 96 or 128: 145 x 136 1219 -> 972.
+// 160^3 x 8 two tiles of 96 columns 117, three of 64 131, and x 12 two of 96 158, of
+// 80 154; 192^3 x 16 x 2 volumes three tiles of 64 columns 338, two of 96 406.  A
+// wider stride than the tile needs takes the second CTA or the attenuation
+// buffer: 132 x 44 x 15 stride 33 two CTAs 47.4, 65 one of 256 threads 54.5, one of
+// 512 51.8; 80 x 96 x 12 stride 49 two CTAs 24.9, 65 one of 256 28.6, one of 512
+// 26.7; 190 x 56 x 12 stride 33 with the buffer 103, 65 without 173.  Planes of 129
+// to 192 columns whole, with the buffer, where they had been two tiles of up to
+// 128 (96 angles, us; in brackets with tiles of any width as before the strides
+// were fixed): 57 x 144 308 -> 180 [186], 76 x 160 470 -> 285 [303], 102 x 136 588
+// -> 424 [426]; two equal tiles of 80 columns in place of 96 or 128: 145 x 136 1219
+// -> 972.
 BackTiling back_tiling(int n, int nz, int rmax, bool atten, size_t limit)
 {
     BackTiling best{};
